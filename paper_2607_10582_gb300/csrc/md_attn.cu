@@ -44,6 +44,8 @@
 
 namespace md {
 
+constexpr int NCW_DEFAULT = 4;
+
 template <int PS, int NCW>
 struct AttnShape {
   static constexpr int NT = PS / 16;                 // 16-token tiles per page
@@ -54,7 +56,8 @@ struct AttnShape {
   static constexpr int RING_BYTES = R * STAGE_BYTES;
   static constexpr int CTAS_PER_SM = 2;
   static constexpr int THREADS = 32 * (NCW + 2);     // producer, NCW consumers, finisher
-  static constexpr int Q_BYTES = GP * D * 2;         // one unit's query heads
+  static constexpr int NEW_OFF = GP * D * 2;         // one unit's query heads, then the
+  static constexpr int Q_BYTES = NEW_OFF + 2 * D * 2;   // new token's K row and V row
   static constexpr int MAX_UNIT_PAGES = MD_MAX_CHUNK_TOKENS / PS;
   static constexpr int MERGE_FLOATS = NCW * (24 + GP * D);
   static constexpr int FIN_FLOATS = 16 + 3 * MD_MAX_CHUNKS * GP;
@@ -94,20 +97,32 @@ __device__ __forceinline__ Unit decode_unit(const AttnParams &p, int u) {
   return un;
 }
 
+/* NEW (a template parameter below): this launch appends the step's new tokens.
+ * Free-stack index of sequence b's last page when the step opens it, or -1:
+ * the block table holds every page. */
+template <bool NEW>
+__device__ __forceinline__ int tail_pop(const AttnParams &p, int b) {
+  return NEW ? p.nt.tail_pop[b] : -1;
+}
+
 /* Physical ids (and, with region-aligned pages, fills) of pages [from,
  * min(from + 8, to)) of unit x; returns how many.  The loads are
  * independent, so all of them are in flight at once. */
-template <bool ALIGNED>
+template <bool ALIGNED, bool NEW>
 __device__ __forceinline__ int load_batch(const AttnParams &p, const Unit &x, int from, int to, int (&ph)[8],
                                           int (&fl)[8]) {
   const int cnt = min(8, to - from);
   const int32_t *bt = p.block_table + (size_t)x.b * p.P_max;
+  const int last = p.n_pages[x.b] - 1;
+  const int pop = tail_pop<NEW>(p, x.b);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) ph[k] = k < cnt ? bt[from + k] : 0;
+  for (int k = 0; k < 8; ++k)
+    ph[k] = k < cnt ? *(pop >= 0 && from + k == last ? p.nt.free_stack + pop : bt + from + k) : 0;
   if (ALIGNED) {
     const uint8_t *fr = p.page_fill + (size_t)x.b * p.P_max;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) fl[k] = k < cnt ? fr[from + k] : 0;
+    for (int k = 0; k < 8; ++k)
+      fl[k] = k >= cnt ? 0 : (NEW && from + k == last ? p.nt.tail_fill[x.b] : fr[from + k]);
   } else {
 #pragma unroll
     for (int k = 0; k < 8; ++k) fl[k] = 0;
@@ -164,20 +179,24 @@ __device__ __forceinline__ void fin_sync() {
 
 /* The unit's physical page ids (and, with region-aligned pages, their fills)
  * into shared memory, loaded in batches. */
-template <bool ALIGNED, int NT>
+template <bool ALIGNED, bool NEW, int NT>
 __device__ __forceinline__ void load_page_ids(const AttnParams &p, const Unit &pv, int tid,
                                               const FinSmem &f) {
   const int npg = pv.p1 - pv.p0;
   const int32_t *bt = p.block_table + (size_t)pv.b * p.P_max;
+  const int last = p.n_pages[pv.b] - 1;
+  const int pop = tail_pop<NEW>(p, pv.b);
   for (int q0 = 0; q0 < npg; q0 += NT * 4) {
     int ph[4], fl[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int q = q0 + r * NT + tid;
+      const bool tail = pv.p0 + q == last;
       ph[r] = fl[r] = 0;
       if (q < npg) {
-        ph[r] = bt[pv.p0 + q];
-        if (ALIGNED) fl[r] = p.page_fill[(size_t)pv.b * p.P_max + pv.p0 + q];
+        ph[r] = *(tail && pop >= 0 ? p.nt.free_stack + pop : bt + pv.p0 + q);
+        if (ALIGNED)
+          fl[r] = NEW && tail ? p.nt.tail_fill[pv.b] : p.page_fill[(size_t)pv.b * p.P_max + pv.p0 + q];
       }
     }
 #pragma unroll
@@ -189,6 +208,38 @@ __device__ __forceinline__ void load_page_ids(const AttnParams &p, const Unit &p
       }
     }
   }
+}
+
+/* One warp puts the new token's K and V rows (row_src: K then V, 256 bytes
+ * each, in shared memory; 16 bytes per lane) into the pool and over their
+ * stale copy in the stage that holds the sequence's last page, at token
+ * `off`; lane 0 of the first layer's KV head 0 starts the token's state. */
+template <int PS>
+__device__ __forceinline__ void append_row(const AttnParams &p, int b, int l, int kvh, int off,
+                                           const uint8_t *row_src, uint8_t *ring, uint32_t ring_u32,
+                                           uint32_t st, int lane) {
+  const int last = p.n_pages[b] - 1;
+  const int pop = tail_pop<true>(p, b);
+  const int phys = pop >= 0 ? p.nt.free_stack[pop] : p.block_table[(size_t)b * p.P_max + last];
+  const uint4 v = *(const uint4 *)(row_src + lane * 16);
+  const int row = (lane < 16 ? 0 : PS) + off;
+  const int d = (lane & 15) * 8;
+  *(uint4 *)(ring + (swz<PS>(st, row, d) - ring_u32)) = v;
+  *(uint4 *)(p.nt.pool + ((((size_t)l * p.P_phys + phys) * p.Hkv + kvh) * 2 * PS + row) * D + d) = v;
+  if (p.nt.init_state && l == p.l0 && kvh == 0 && lane == 0) {
+    const size_t slot = (size_t)phys * PS + off;
+    p.nt.region[slot] = p.nt.tail_region[b];
+    p.nt.t_ref[slot] = p.nt.insert_step;
+    p.nt.t_ins[slot] = p.nt.insert_step;
+    p.nt.a[slot] = 0.f;
+    p.nt.window[slot] = 0.f;
+    p.nt.ahat[slot] = 0.f;
+    p.nt.prio[slot] = 0.f;
+    if (pop >= 0) p.nt.block_table[(size_t)b * p.P_max + last] = phys;
+    p.nt.page_fill[(size_t)b * p.P_max + last] = (uint8_t)(off + 1);
+    p.nt.seq_tokens[b] += 1;
+  }
+  __syncwarp();
 }
 
 /* Token masses of a unit from its stored raw scores and the item's per-head
@@ -253,14 +304,14 @@ __device__ __forceinline__ void mass_pass(const AttnParams &p, const Unit &pv, i
  * warp, or all consumer warps for a CTA's last unit.  Returns false, the same
  * for every thread, on abort or timeout.  Loads are issued in batches before
  * the dependent stores, so a pass costs a few L2 round trips. */
-template <int PS, bool ALIGNED, int NT, int OBUF_FLOATS, bool ROWS>
+template <int PS, bool ALIGNED, int NT, int OBUF_FLOATS, bool ROWS, bool NEW>
 __device__ __forceinline__ bool finish_unit(const AttnParams &p, const Unit &pv, int slot, int tid,
                                             const FinSmem &f) {
   const float NEG_INF = -INFINITY;
   const int G = p.G;
   const int C = pv.C;
   /* the unit's page ids (no wait needed) */
-  load_page_ids<ALIGNED, NT>(p, pv, tid, f);
+  load_page_ids<ALIGNED, NEW, NT>(p, pv, tid, f);
   /* all chunks of the item published */
   if (tid == 0) {
     int okw = 1;
@@ -452,11 +503,11 @@ __device__ __forceinline__ void merge_single(const AttnParams &p, const Unit &un
 /* The whole end of a single-chunk unit: the page ids, the merge straight
  * into (max, 1/Z) and the output, the release of the merge buffers (mdone,
  * when given: the finisher's hand-off), the token masses. */
-template <int PS, bool ALIGNED, int NCW, int NT, bool ROWS>
+template <int PS, bool ALIGNED, int NCW, int NT, bool ROWS, bool NEW>
 __device__ __forceinline__ void single_end(const AttnParams &p, const Unit &un, int slot, int tid,
                                         const float *wm, const float *wl, float *wf,
                                         const float *wO, const FinSmem &f, uint32_t mdone) {
-  load_page_ids<ALIGNED, NT>(p, un, tid, f);
+  load_page_ids<ALIGNED, NEW, NT>(p, un, tid, f);
   merge_single<NCW, NT>(p, un, tid, wm, wl, wf, wO, f);
   if (mdone != 0 && tid == 0) mbar_arrive(mdone);   // merge buffers free again
   mass_pass<PS, ALIGNED, NT, ROWS>(p, un, slot, tid, f);
@@ -466,9 +517,12 @@ __device__ __forceinline__ void single_end(const AttnParams &p, const Unit &un, 
 /* ALIGNED: pages carry their own fill (region-aligned allocation); otherwise
  * every page but the last is full and the fills follow from n_tokens.  ROWS:
  * the masses go to one fp32 row per (layer, KV head) (the no-allocation entry
- * point) instead of the step's fixed-point accumulator; a compile-time choice,
- * since this end-of-unit code runs once per unit and is often fetched cold. */
-template <int PS, int NCW, bool ALIGNED, bool ROWS>
+ * point) instead of the step's fixed-point accumulator.  NEW: the launch
+ * also appends the step's new tokens (NewTokens).  Compile-time choices: the
+ * end-of-unit code runs once per unit and is often fetched cold, and a runtime
+ * test in the page loads made the no-allocation call 3% longer (24 x 999
+ * tokens, 16 layers: 60.6 -> 62.5 us). */
+template <int PS, int NCW, bool ALIGNED, bool ROWS, bool NEW>
 __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW>::CTAS_PER_SM)
     attn_mass_kernel(const __grid_constant__ AttnParams p,
                      const __grid_constant__ CUtensorMap tmap) {
@@ -554,6 +608,9 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
       int ph[8], fl[8];
       if (u < p.total_units) {
         un = decode_unit(p, u);
+        pb = un.p0;
+      }
+      if (u < p.total_units && !NEW) {
         /* before the wait: the first unit's query rows (the caller's) and,
          * when the unit is its item's only chunk, its pages below the
          * sequence's last one, at most one per stage (measured on a GB300:
@@ -565,7 +622,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
         nu = 1;
         const int early_end = un.C == 1 ? min(min(un.p1, un.p0 + S::R), p.n_pages[un.b] - 1) : un.p0;
         for (pb = un.p0; pb < early_end; pb += 8) {
-          cnt = load_batch<ALIGNED>(p, un, pb, early_end, ph, fl);
+          cnt = load_batch<ALIGNED, NEW>(p, un, pb, early_end, ph, fl);
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
             if (k >= cnt) break;
@@ -583,7 +640,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
       }
       pdl_wait();
       pdl_trigger();
-      if (u < p.total_units) cnt = pb < un.p1 ? load_batch<ALIGNED>(p, un, pb, un.p1, ph, fl) : 0;
+      if (u < p.total_units) cnt = pb < un.p1 ? load_batch<ALIGNED, NEW>(p, un, pb, un.p1, ph, fl) : 0;
       while (u < p.total_units && ok) {
         Unit nx = un;
         int npb = pb + 8, nxu = u, cntn = 0;
@@ -595,9 +652,10 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
             npb = nx.p0;
           }
         }
-        if (nxu < p.total_units) cntn = load_batch<ALIGNED>(p, nx, npb, nx.p1, phn, fln);
-        if (pb == un.p0 && u != (int)blockIdx.x) {   // the first unit's rows went out before the wait
-          /* the unit's G query rows: one bulk copy into a double-buffered slot */
+        if (nxu < p.total_units) cntn = load_batch<ALIGNED, NEW>(p, nx, npb, nx.p1, phn, fln);
+        if (pb == un.p0 && (NEW || u != (int)blockIdx.x)) {   // not NEW: the first unit's went out before the wait
+          /* the unit's G query rows (and the new token's K and V rows, where
+           * the unit holds its page) into a double-buffered slot */
           const int qs = nu & 1;
           if (nu >= 2) {
             if (!wait_phase(smem_u32(&qempty[qs]), ((nu >> 1) - 1) & 1, p, 5, true)) {
@@ -608,10 +666,17 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
              * copy writes it through the async proxy */
             fence_proxy_async_smem();
           }
-          mbar_arrive_expect_tx(smem_u32(&qfull[qs]), G * D * 2);
+          const bool tail = NEW && un.p1 == p.n_pages[un.b];
+          mbar_arrive_expect_tx(smem_u32(&qfull[qs]), G * D * 2 + (tail ? 2 * D * 2 : 0));
           bulk_load(sQ_u32 + qs * S::Q_BYTES,
                     p.q + (((size_t)un.b * p.q_layers + (un.l - p.l0)) * p.Hq + (size_t)un.kvh * G) * D,
                     G * D * 2, smem_u32(&qfull[qs]));
+          if (tail) {
+            const long long src = un.b * p.nt.sb + (un.l - p.l0) * p.nt.sl + un.kvh * D;
+            const uint32_t dst = sQ_u32 + qs * S::Q_BYTES + S::NEW_OFF;
+            bulk_load(dst, p.nt.k_new + src, D * 2, smem_u32(&qfull[qs]));
+            bulk_load(dst + D * 2, p.nt.v_new + src, D * 2, smem_u32(&qfull[qs]));
+          }
           ++nu;
         }
 #pragma unroll
@@ -671,11 +736,11 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
       const bool ok = wait_phase(smem_u32(&cdone[k & 1]), (k >> 1) & 1, p, 8, true);
       if (!__all_sync(0xffffffffu, ok)) break;
       if (pv.C == 1) {
-        single_end<PS, ALIGNED, NCW, 32, ROWS>(p, pv, k & 1, lane, wm, wl, wf, wO, fs, smem_u32(&mdone[0]));
+        single_end<PS, ALIGNED, NCW, 32, ROWS, NEW>(p, pv, k & 1, lane, wm, wl, wf, wO, fs, smem_u32(&mdone[0]));
       } else {
         merge_publish<NCW, 32>(p, pv, lane, wm, wl, wf, wO);
         if (lane == 0) mbar_arrive(smem_u32(&mdone[0]));   // merge buffers free again
-        if (!finish_unit<PS, ALIGNED, 32, S::OBUF_FLOATS, ROWS>(p, pv, k & 1, lane, fs)) break;
+        if (!finish_unit<PS, ALIGNED, 32, S::OBUF_FLOATS, ROWS, NEW>(p, pv, k & 1, lane, fs)) break;
       }
       if (lane == 0) mbar_arrive(smem_u32(&fdone[k & 1]));   // slot and finish area free
     }
@@ -697,6 +762,15 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
     const Unit un = decode_unit(p, u);
     const int npg = un.p1 - un.p0;
     const int slot = nunit & 1;
+    /* this warp's pages are those whose CTA-wide index gi = i_base + jp is
+     * cw modulo NCW: they land only in this warp's own stages (gi % R), so a
+     * wait is never more than one phase ahead of the copies however far the
+     * warps drift apart, and a unit's extra pages rotate over the warps */
+    const int j0 = ((cw - i_base) % NCW + NCW) % NCW;
+    /* the page the new token goes on, when this warp has it (else -1): the
+     * warp then keeps the query slot, which also holds the token's rows */
+    int jtail = NEW ? p.n_pages[un.b] - 1 - un.p0 : -1;
+    if (NEW && (jtail >= npg || (jtail - j0) % NCW != 0)) jtail = -1;
     float *scr = p.scratch + ((size_t)blockIdx.x * 2 + slot) * p.scratch_tokens * GP;
 
     /* Q^T fragments (B operand) from the prefetched rows: head g, dims
@@ -718,7 +792,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
         qf[kk + 1][1] = gv ? r3 : 0u;
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&qempty[qs]));
+      if ((!NEW || jtail < 0) && lane == 0) mbar_arrive(smem_u32(&qempty[qs]));
     }
     /* the score slot is free once the finisher is done with the unit that
      * used it two units ago */
@@ -733,11 +807,6 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
     const int ntok_seq = p.n_tokens[un.b];
     const int mi = lane >> 3, rr = lane & 7;
 
-    /* this warp's pages are those whose CTA-wide index gi = i_base + jp is
-     * cw modulo NCW: they land only in this warp's own stages (gi % R), so a
-     * wait is never more than one phase ahead of the copies however far the
-     * warps drift apart, and a unit's extra pages rotate over the warps */
-    const int j0 = ((cw - i_base) % NCW + NCW) % NCW;
     for (int jp = j0; jp < npg && !aborted; jp += NCW) {
       const int gi = i_base + jp;
       const int s = gi % S::R;
@@ -747,6 +816,9 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
       }
       const uint32_t st = ring_u32 + s * S::STAGE_BYTES;
       const int fill = ALIGNED ? fillbuf[s] : ntok_seq - (un.p0 + jp) * PS;
+      if (NEW && jp == jtail)
+        append_row<PS>(p, un.b, un.l, un.kvh, fill - 1, sQ + (nunit & 1) * S::Q_BYTES + S::NEW_OFF, ring,
+                       ring_u32, st, lane);
 
       float acc[S::NT][4];
 #pragma unroll
@@ -816,6 +888,8 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
       if (lane == 0) mbar_arrive(smem_u32(&empty[s]));
     }
 
+    if (NEW && jtail >= 0 && lane == 0) mbar_arrive(smem_u32(&qempty[nunit & 1]));
+
     /* ---- the unit's end: this warp's softmax state goes to the merge ---- */
 #pragma unroll
     for (int off = 4; off < 32; off <<= 1) {
@@ -864,90 +938,99 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
     named_barrier(1, NC);
     if (flag[0]) break;
     if (un.C == 1) {
-      single_end<PS, ALIGNED, NCW, NCW * 32, ROWS>(p, un, slot, ct, wm, wl, wf, wO, fs, 0u);
+      single_end<PS, ALIGNED, NCW, NCW * 32, ROWS, NEW>(p, un, slot, ct, wm, wl, wf, wO, fs, 0u);
       break;
     }
     merge_publish<NCW, NCW * 32>(p, un, ct, wm, wl, wf, wO);
     if (ct == 0) flag[1] = ld_volatile(&p.status[ST_ABORT]);
     named_barrier(1, NC);
     if (flag[1]) break;
-    finish_unit<PS, ALIGNED, NCW * 32, S::OBUF_FLOATS, ROWS>(p, un, slot, ct, fs);
+    finish_unit<PS, ALIGNED, NCW * 32, S::OBUF_FLOATS, ROWS, NEW>(p, un, slot, ct, fs);
     break;
   }
 }
 
-template <int PS, int NCW, bool AL, bool ROWS>
+template <int PS, bool AL, bool ROWS, bool NEW>
 static cudaError_t prepare_impl() {
-  return cudaFuncSetAttribute(attn_mass_kernel<PS, NCW, AL, ROWS>,
+  return cudaFuncSetAttribute(attn_mass_kernel<PS, NCW_DEFAULT, AL, ROWS, NEW>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)AttnShape<PS, NCW>::SMEM);
+                              (int)AttnShape<PS, NCW_DEFAULT>::SMEM);
 }
 
 /* The instances of one page size: the step's (contiguous or region-aligned
- * pages) and the no-allocation entry point's (contiguous pages, mass rows). */
-template <int PS, int NCW>
+ * pages, with or without the append) and the no-allocation entry point's
+ * (contiguous pages, mass rows). */
+template <int PS>
 static cudaError_t prepare_all() {
-  cudaError_t e = prepare_impl<PS, NCW, false, false>();
-  if (e == cudaSuccess) e = prepare_impl<PS, NCW, true, false>();
-  if (e == cudaSuccess) e = prepare_impl<PS, NCW, false, true>();
+  cudaError_t e = prepare_impl<PS, false, false, false>();
+  if (e == cudaSuccess) e = prepare_impl<PS, true, false, false>();
+  if (e == cudaSuccess) e = prepare_impl<PS, false, false, true>();
+  if (e == cudaSuccess) e = prepare_impl<PS, true, false, true>();
+  if (e == cudaSuccess) e = prepare_impl<PS, false, true, false>();
   return e;
 }
 
-template <int PS, int NCW>
+template <int PS>
 static int grid_limit_impl() {
-  int dev = 0, sms = 0, per_sm = 0;
+  using S = AttnShape<PS, NCW_DEFAULT>;
+  int dev = 0, sms = 0, per_sm = 0, per_sm_new = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (prepare_all<PS, NCW>() != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, attn_mass_kernel<PS, NCW, false, false>,
-                                                    AttnShape<PS, NCW>::THREADS,
-                                                    AttnShape<PS, NCW>::SMEM) != cudaSuccess)
+  if (prepare_all<PS>() != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, attn_mass_kernel<PS, NCW_DEFAULT, false, false, false>,
+                                                    S::THREADS, S::SMEM) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_new, attn_mass_kernel<PS, NCW_DEFAULT, false, false, true>,
+                                                    S::THREADS, S::SMEM) != cudaSuccess)
     return 0;
-  int g = sms * per_sm;
+  int g = sms * (per_sm < per_sm_new ? per_sm : per_sm_new);
   return g > MAX_GRID ? MAX_GRID : g;
 }
 
-template <int PS, int NCW, bool AL, bool ROWS>
-static cudaError_t launch_impl(const AttnParams &p, const CUtensorMap &tmap, int grid,
-                               cudaStream_t s) {
+/* Launches whose items are all single chunks have no cross-CTA waits and need
+ * no co-residency: without the cooperative attribute a chain of dependent
+ * launches costs 1.7 us per launch on the GPU instead of 3.1. */
+template <int PS, bool AL, bool ROWS, bool NEW>
+static cudaError_t launch_impl(const AttnParams &p, const CUtensorMap &tmap, int grid, cudaStream_t s) {
+  using S = AttnShape<PS, NCW_DEFAULT>;
+  bool split = ROWS;   // the no-allocation call follows a memset: 59.8 us with, 61.2 us without the attribute
+  for (int b = 0; b < p.n_seqs; ++b) split |= p.chunks[b] > 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(AttnShape<PS, NCW>::THREADS);
-  cfg.dynamicSmemBytes = AttnShape<PS, NCW>::SMEM;
+  cfg.blockDim = dim3(S::THREADS);
+  cfg.dynamicSmemBytes = S::SMEM;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeCooperative;
+  attr[1].val.cooperative = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, attn_mass_kernel<PS, NCW, AL, ROWS>, p, tmap);
+  cfg.numAttrs = split ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, attn_mass_kernel<PS, NCW_DEFAULT, AL, ROWS, NEW>, p, tmap);
 }
 
-constexpr int NCW_DEFAULT = 4;
+cudaError_t attention_prepare(int ps) { return ps == 16 ? prepare_all<16>() : prepare_all<32>(); }
 
-cudaError_t attention_prepare(int ps) {
-  return ps == 16 ? prepare_all<16, NCW_DEFAULT>() : prepare_all<32, NCW_DEFAULT>();
-}
+int attention_grid_limit(int ps) { return ps == 16 ? grid_limit_impl<16>() : grid_limit_impl<32>(); }
 
-int attention_grid_limit(int ps) {
-  return ps == 16 ? grid_limit_impl<16, NCW_DEFAULT>() : grid_limit_impl<32, NCW_DEFAULT>();
+template <int PS>
+static cudaError_t launch_ps(const AttnParams &p, const CUtensorMap &tmap, int grid, cudaStream_t s) {
+  const bool add = p.nt.free_stack != nullptr;
+  if (!p.mass_acc) {   // mass rows: the no-allocation entry point, contiguous pages
+    if (p.page_fill || add) return cudaErrorInvalidValue;
+    return launch_impl<PS, false, true, false>(p, tmap, grid, s);
+  }
+  if (p.page_fill)
+    return add ? launch_impl<PS, true, false, true>(p, tmap, grid, s)
+               : launch_impl<PS, true, false, false>(p, tmap, grid, s);
+  return add ? launch_impl<PS, false, false, true>(p, tmap, grid, s)
+             : launch_impl<PS, false, false, false>(p, tmap, grid, s);
 }
 
 cudaError_t launch_attention(const AttnParams &p, const CUtensorMap &tmap, int grid,
                              cudaStream_t s) {
   if (p.total_units == 0) return cudaSuccess;
-  if (!p.mass_acc) {   // mass rows: the no-allocation entry point, contiguous pages
-    if (p.page_fill) return cudaErrorInvalidValue;
-    return p.ps == 16 ? launch_impl<16, NCW_DEFAULT, false, true>(p, tmap, grid, s)
-                      : launch_impl<32, NCW_DEFAULT, false, true>(p, tmap, grid, s);
-  }
-  if (p.page_fill)
-    return p.ps == 16 ? launch_impl<16, NCW_DEFAULT, true, false>(p, tmap, grid, s)
-                      : launch_impl<32, NCW_DEFAULT, true, false>(p, tmap, grid, s);
-  return p.ps == 16 ? launch_impl<16, NCW_DEFAULT, false, false>(p, tmap, grid, s)
-                    : launch_impl<32, NCW_DEFAULT, false, false>(p, tmap, grid, s);
+  return p.ps == 16 ? launch_ps<16>(p, tmap, grid, s) : launch_ps<32>(p, tmap, grid, s);
 }
 
 }  // namespace md

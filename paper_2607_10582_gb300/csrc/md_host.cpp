@@ -59,6 +59,7 @@ struct md_ctx {
   std::vector<int> n_pages, pinned_pages;
   std::vector<int> tail_fill, tail_region;  // the page being written
   std::vector<uint8_t> tail_pinned, tokens_exact;
+  std::vector<int> tail_pop;   // this decode step: free-stack index of the page each new token opens, or -1
   bool poisoned = false;
   std::string err;
   long long spin_limit_ns = 2000000000LL;
@@ -183,13 +184,6 @@ int evictable_pages(const md_ctx *c, int b) {
 bool opens_page(const md_ctx *c, int b, int r) {
   return c->n_pages[b] == 0 || c->tail_fill[b] == c->cfg.page_size ||
          (c->cfg.region_aligned_pages && c->tail_region[b] != r);
-}
-
-/* Slot (page * page_size + offset, in logical page order) the next token of
- * region r goes to. */
-int next_slot(const md_ctx *c, int b, int r) {
-  const int ps = c->cfg.page_size;
-  return opens_page(c, b, r) ? c->n_pages[b] * ps : (c->n_pages[b] - 1) * ps + c->tail_fill[b];
 }
 
 /* Mirror bookkeeping for one appended token of region r. */
@@ -552,6 +546,7 @@ MD_API md_status md_create(const md_config *cfg, md_ctx **out) {
   c->tail_fill.assign(B, 0);
   c->tail_region.assign(B, -1);
   c->tokens_exact.assign(B, 1);
+  c->tail_pop.assign(B, -1);
   for (int r = 0; r < 8; ++r) {
     c->reg.base[r] = 0.f;
     c->reg.half_life[r] = INFINITY;
@@ -717,9 +712,6 @@ MD_API md_status md_append_tokens(md_ctx *c, int seq, int n, const uint8_t *regi
   ap.ps = ps;
   ap.P_phys = cf.num_phys_pages;
   ap.P_max = cf.max_pages_per_seq;
-  ap.l0 = 0;
-  ap.init_state = 1;
-  ap.lookup_only = 0;
   ap.n_seqs = 1;
   ap.n_per_seq = n;
   ap.seq0 = seq;
@@ -783,51 +775,58 @@ void fill_append_common(md_ctx *c, AppendParams &ap) {
   ap.seq0 = 0;
 }
 
-/* Start of a decode step: advance t, take the new pages, append the new
- * tokens' K/V for layers [l0, l0 + L) and start their state. */
-md_status begin_step(md_ctx *c, int batch, int l0, int L, long long sb, long long sl,
-                     const void *k_new, const void *v_new, const uint8_t *new_region_host) {
-  const int ps = c->cfg.page_size;
+/* Start of a decode step: fold the step before it, advance t, take the new
+ * tokens' pages.  The append launch or the attention launch then writes the
+ * rows and the tokens' state. */
+md_status begin_step(md_ctx *c, int batch, const uint8_t *new_region_host) {
   if (c->m.mass_pending) {
     md_status st = launch_fold(c);
     if (st != MD_OK) return st;
   }
   c->m.t += 1;
+  int64_t top = c->m.free_top;
+  for (int b = 0; b < batch; ++b) {
+    c->tail_pop[b] = opens_page(c, b, new_region_host[b]) ? (int)--top : -1;
+    mirror_token(c, b, new_region_host[b]);
+  }
+  c->m.free_top = top;
+  return MD_OK;
+}
+
+/* The step's append as a launch of its own, for new K/V that lie in host
+ * memory: every layer's rows in one pass over the host link, where the
+ * attention units' reads of two short rows each would pay its latency. */
+md_status append_step(md_ctx *c, int batch, const void *k_new, const void *v_new) {
+  const md_config &cf = c->cfg;
   AppendParams ap;
   fill_append_common(c, ap);
   ap.k_src = (const uint16_t *)k_new;
   ap.v_src = (const uint16_t *)v_new;
-  ap.sb = sb;
-  ap.sl = sl;
+  ap.sb = (long long)cf.num_layers * cf.num_kv_heads * D;
+  ap.sl = (long long)cf.num_kv_heads * D;
   ap.sh = D;
   ap.si = 0;
-  ap.L = L;
-  ap.l0 = l0;
-  ap.init_state = 1;
-  ap.lookup_only = 0;
+  ap.L = cf.num_layers;
   ap.n_seqs = batch;
   ap.insert_step = (int)c->m.t;
-  long long popped = 0;
   for (int b = 0; b < batch; ++b) {
-    ap.tok0[b] = next_slot(c, b, new_region_host[b]);
-    ap.pages_before[b] = c->n_pages[b];
-    ap.pop_base[b] = (int)(c->m.free_top - 1 - popped);
-    ap.regions_param[b] = new_region_host[b];
-    if (opens_page(c, b, new_region_host[b])) popped += 1;
+    const bool opened = c->tail_pop[b] >= 0;
+    ap.tok0[b] = (c->n_pages[b] - 1) * cf.page_size + c->tail_fill[b] - 1;
+    ap.pages_before[b] = c->n_pages[b] - (opened ? 1 : 0);
+    ap.pop_base[b] = c->tail_pop[b];
+    ap.regions_param[b] = (uint8_t)c->tail_region[b];
   }
   cudaEvent_t e0;
   prof_begin(c, &e0);
   cudaError_t e = launch_append(ap, c->stream);
   prof_end(c, STAGE_APPEND, e0);
-  if (e != cudaSuccess) return cuda_fail(c, e, "append launch");
-  for (int b = 0; b < batch; ++b) mirror_token(c, b, new_region_host[b]);
-  c->m.free_top -= popped;
-  return MD_OK;
+  return e == cudaSuccess ? MD_OK : cuda_fail(c, e, "append launch");
 }
 
-/* Stage 1 over layers [l0, l0 + L); q/out hold q_layers layers. */
+/* Stage 1 over layers [l0, l0 + L); q/out hold q_layers layers.  With k_new
+ * the launch also appends the step's new tokens (device rows [batch][L][Hkv][D]). */
 md_status run_attention(md_ctx *c, int batch, int l0, int L, int q_layers, const void *q_dev,
-                        void *out_dev) {
+                        const void *k_new, const void *v_new, void *out_dev) {
   const md_config &cf = c->cfg;
   AttnParams atp;
   memset(&atp, 0, sizeof(atp));
@@ -857,6 +856,32 @@ md_status run_attention(md_ctx *c, int batch, int l0, int L, int q_layers, const
   atp.spin_limit_ns = c->spin_limit_ns;
   atp.extra_arrivals = c->extra_arrivals;
   c->extra_arrivals = 0;
+  if (k_new) {
+    NewTokens &nt = atp.nt;
+    nt.k_new = (const uint16_t *)k_new;
+    nt.v_new = (const uint16_t *)v_new;
+    nt.sb = (long long)L * cf.num_kv_heads * D;
+    nt.sl = (long long)cf.num_kv_heads * D;
+    nt.pool = ptr<uint16_t>(c, c->lay.pool);
+    nt.free_stack = ptr<int32_t>(c, c->lay.free_stack);
+    nt.block_table = ptr<int32_t>(c, c->lay.block_table);
+    nt.region = ptr<uint8_t>(c, c->lay.region);
+    nt.page_fill = ptr<uint8_t>(c, c->lay.page_fill);
+    nt.t_ref = ptr<int32_t>(c, c->lay.t_ref);
+    nt.t_ins = ptr<int32_t>(c, c->lay.t_ins);
+    nt.seq_tokens = ptr<int32_t>(c, c->lay.seq_tokens);
+    nt.a = ptr<float>(c, c->lay.a);
+    nt.window = ptr<float>(c, c->lay.window);
+    nt.ahat = ptr<float>(c, c->lay.ahat);
+    nt.prio = ptr<float>(c, c->lay.prio);
+    nt.init_state = l0 == 0;
+    nt.insert_step = (int)c->m.t;
+    for (int b = 0; b < batch; ++b) {
+      nt.tail_pop[b] = c->tail_pop[b];
+      nt.tail_fill[b] = (uint8_t)c->tail_fill[b];
+      nt.tail_region[b] = (uint8_t)c->tail_region[b];
+    }
+  }
   int grid = 1;
   plan_attention(c, batch, L, atp, &grid);
   cudaEvent_t e0;
@@ -877,19 +902,6 @@ void end_step(md_ctx *c, int batch) {
 }  // namespace
 
 namespace {
-
-/* The whole decode step once its arguments are checked. */
-md_status decode_step_core(md_ctx *c, int batch, const void *q, const void *k_new, const void *v_new,
-                           const uint8_t *new_region_host, void *out) {
-  const md_config &cf = c->cfg;
-  md_status st = begin_step(c, batch, 0, cf.num_layers, (long long)cf.num_layers * cf.num_kv_heads * D,
-                            (long long)cf.num_kv_heads * D, k_new, v_new, new_region_host);
-  if (st != MD_OK) return st;
-  st = run_attention(c, batch, 0, cf.num_layers, cf.num_layers, q, out);
-  if (st != MD_OK) return st;
-  end_step(c, batch);
-  return MD_OK;
-}
 
 /* The address at which the kernels can use host buffer h directly, or null:
  * pinned (page-locked) or registered memory at its device address, any other
@@ -919,7 +931,11 @@ MD_API md_status md_decode_step(md_ctx *c, int batch, const void *q_dev, const v
   if (!q_dev || !k_new || !v_new || !out_dev) return fail(c, MD_ERR_INVALID_ARG, "null pointer");
   md_status st = check_step(c, batch, new_region_host);
   if (st != MD_OK) return st;
-  return decode_step_core(c, batch, q_dev, k_new, v_new, new_region_host, out_dev);
+  st = begin_step(c, batch, new_region_host);
+  if (st != MD_OK) return st;
+  st = run_attention(c, batch, 0, c->cfg.num_layers, c->cfg.num_layers, q_dev, k_new, v_new, out_dev);
+  if (st == MD_OK) end_step(c, batch);
+  return st;
 }
 
 MD_API md_status md_decode_step_host(md_ctx *c, int batch, const void *q_host, const void *k_new_host,
@@ -954,8 +970,13 @@ MD_API md_status md_decode_step_host(md_ctx *c, int batch, const void *q_host, c
   if (e == cudaSuccess && !vk) e = cudaMemcpyAsync(dk, k_new_host, kv_bytes, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess && !vv) e = cudaMemcpyAsync(dv, v_new_host, kv_bytes, cudaMemcpyHostToDevice, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "input copy");
-  st = decode_step_core(c, batch, dq, vk ? vk : dk, vv ? vv : dv, new_region_host, vo ? vo : dout);
+  st = begin_step(c, batch, new_region_host);
   if (st != MD_OK) return st;
+  st = append_step(c, batch, vk ? vk : dk, vv ? vv : dv);
+  if (st != MD_OK) return st;
+  st = run_attention(c, batch, 0, cf.num_layers, cf.num_layers, dq, nullptr, nullptr, vo ? vo : dout);
+  if (st != MD_OK) return st;
+  end_step(c, batch);
   if (!vo) {
     e = cudaMemcpyAsync(out_host, dout, q_bytes, cudaMemcpyDeviceToHost, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "output copy");
@@ -976,36 +997,13 @@ MD_API md_status md_decode_layer(md_ctx *c, int layer, int batch, const void *q_
   if (layer == 0) {
     st = check_step(c, batch, new_region_host);
     if (st != MD_OK) return st;
-    st = begin_step(c, batch, 0, 1, (long long)cf.num_kv_heads * D, 0, k_new, v_new,
-                    new_region_host);
+    st = begin_step(c, batch, new_region_host);
     if (st != MD_OK) return st;
     c->m.layer_batch = batch;
-  } else {
-    if (batch != c->m.layer_batch)
-      return fail(c, MD_ERR_INVALID_ARG, "batch changed within a decode step");
-    /* the new tokens' pages and state exist: write this layer's K/V only */
-    AppendParams ap;
-    fill_append_common(c, ap);
-    ap.k_src = (const uint16_t *)k_new;
-    ap.v_src = (const uint16_t *)v_new;
-    ap.sb = (long long)cf.num_kv_heads * D;
-    ap.sl = 0;
-    ap.sh = D;
-    ap.si = 0;
-    ap.L = 1;
-    ap.l0 = layer;
-    ap.init_state = 0;
-    ap.lookup_only = 1;
-    ap.n_seqs = batch;
-    for (int b = 0; b < batch; ++b)
-      ap.tok0[b] = (c->n_pages[b] - 1) * cf.page_size + c->tail_fill[b] - 1;
-    cudaEvent_t e0;
-    prof_begin(c, &e0);
-    cudaError_t e = launch_append(ap, c->stream);
-    prof_end(c, STAGE_APPEND, e0);
-    if (e != cudaSuccess) return cuda_fail(c, e, "append launch");
+  } else if (batch != c->m.layer_batch) {
+    return fail(c, MD_ERR_INVALID_ARG, "batch changed within a decode step");
   }
-  st = run_attention(c, batch, layer, 1, 1, q_dev, out_dev);
+  st = run_attention(c, batch, layer, 1, 1, q_dev, k_new, v_new, out_dev);
   if (st != MD_OK) return st;
   c->m.layer_next = layer + 1;
   if (c->m.layer_next == cf.num_layers) {

@@ -63,7 +63,7 @@ __global__ void append_kernel(const __grid_constant__ AppendParams p) {
     const int seq = p.seq0 + j;
     const int tok = p.slots_dev ? p.slots_dev[i] : p.tok0[j] + i;   // slot in the sequence
     const int pg = tok / p.ps, off = tok - pg * p.ps;
-    const int pages_before = p.lookup_only ? 0x7fffffff : p.pages_before[j];
+    const int pages_before = p.pages_before[j];
     int phys;
     if (pg < pages_before)
       phys = p.block_table[(size_t)seq * p.P_max + pg];
@@ -73,11 +73,11 @@ __global__ void append_kernel(const __grid_constant__ AppendParams p) {
     const uint16_t *src = (kv == 0 ? p.k_src : p.v_src) + (long long)j * p.sb +
                           (long long)l * p.sl + (long long)h * p.sh + (long long)i * p.si;
     uint16_t *dst = p.pool +
-                    ((((size_t)(p.l0 + l) * p.P_phys + phys) * p.Hkv + h) * 2 + kv) * (size_t)p.ps * D +
+                    ((((size_t)l * p.P_phys + phys) * p.Hkv + h) * 2 + kv) * (size_t)p.ps * D +
                     (size_t)off * D;
     ((uint4 *)dst)[c] = ((const uint4 *)src)[c];
 
-    if (p.init_state && c == 0 && kv == 0 && h == 0 && l == 0) {
+    if (c == 0 && kv == 0 && h == 0 && l == 0) {
       const size_t slot = (size_t)phys * p.ps + off;
       p.region[slot] = p.regions_dev ? p.regions_dev[i] : p.regions_param[j];
       p.t_ref[slot] = p.steps_dev ? p.steps_dev[i] : p.insert_step;

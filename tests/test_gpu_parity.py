@@ -407,6 +407,55 @@ def test_entry_points_mixed_step_by_step():
     ls.check_layout()
 
 
+@pytest.mark.parametrize("ps,aligned", [(16, 0), (32, 0), (16, 1), (32, 1)])
+@pytest.mark.parametrize("entry", ["device", "layers"])
+def test_append_inside_attention_writes_what_the_append_kernel_writes(ps, aligned, entry):
+    """Decode steps whose attention launch appends the new tokens leave the
+    same pool, token state and page tables, bit for bit, as steps whose append
+    is a launch of its own (host buffers).  Lengths put the new token on the
+    first and the last slot of a page, on both 16-token tiles of a 32-token
+    page and into an empty sequence; region changes open pages early."""
+    L, Hq, Hkv = 2, 16, 2
+    lengths = [0, 1, ps - 1, ps, ps + 1, 5 * ps - 1, 33 * ps, 700]
+    B = len(lengths)
+    rng = np.random.default_rng(7)
+    caches = [md.Cache(L, Hq, Hkv, ps, B, 64, 64 * B, region_aligned_pages=aligned) for _ in range(2)]
+    regs = [np.sort(rng.integers(0, 7, n)).astype(np.uint8) for n in lengths]
+    for c in caches:
+        for r in range(7):
+            c.set_region_params(r, 1.0, 50.0, r == 0)
+        for b, n in enumerate(lengths):
+            if n:
+                k, v = synth.kv_host(3, b, L, Hkv, 0, n, regs[b])
+                c.append_tokens(b, regs[b], to_dev(k), to_dev(v))
+    for step in range(ps + 2):
+        new = rng.integers(0, 7, B).astype(np.uint8) if step % 3 == 0 else np.full(B, 6, np.uint8)
+        q = synth.q_host(3, B, L, Hq, Hkv, step + 1)
+        kn, vn = synth.step_kv_host(3, [n + step for n in lengths], new, L, Hkv)
+        out = torch.empty((B, L, Hq, 128), dtype=torch.int16, device="cuda")
+        if entry == "device":
+            caches[0].decode_step(B, to_dev(q), to_dev(kn), to_dev(vn), new, out)
+        else:
+            for l in range(L):
+                o = torch.empty((B, Hq, 128), dtype=torch.int16, device="cuda")
+                caches[0].decode_layer(l, B, to_dev(q[:, l]), to_dev(kn[:, l]), to_dev(vn[:, l]), new, o)
+                out[:, l] = o
+        pin = [torch.from_numpy(np.ascontiguousarray(a).view(np.int16)).pin_memory() for a in (q, kn, vn)]
+        out_h = torch.empty((B, L, Hq, 128), dtype=torch.int16).pin_memory()
+        caches[1].decode_step_host(B, *pin, new, out_h)
+        assert caches[1].sync() == md.MD_OK
+        diff = synth.bf16_to_f64(out.cpu().numpy().view(np.uint16)) - synth.bf16_to_f64(out_h.numpy().view(np.uint16))
+        assert np.max(np.abs(diff)) <= TOL_O_ABS
+        if step % 5 == 4:      # an eviction in between: pages are freed and taken again
+            for c in caches:
+                c.evict([max(2, c.query(md.MD_QUERY_PAGES, b) - 2) for b in range(B)])
+        for what in (md.MD_STATE_POOL, md.MD_STATE_REGION, md.MD_STATE_T_INS, md.MD_STATE_BLOCK_TABLE,
+                     md.MD_STATE_PAGE_FILL, md.MD_STATE_SEQ_TOKENS, md.MD_STATE_FREE):
+            assert torch.equal(caches[0].get_state(what), caches[1].get_state(what)), (step, what)
+    for c in caches:
+        c.close()
+
+
 def test_checkpoint_restore_replays_step():
     w = synth.custom_workload("ckpt", L=2, Hq=8, Hkv=2, page_size=16, lengths=[900],
                               budget_frac=0.3, steps=2, seed=9)
