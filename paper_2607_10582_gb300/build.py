@@ -14,7 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB_PATH = os.path.join(HERE, "libmemdecay.so")
 OBJ_DIR = os.path.join(HERE, "_build")
-SOURCES = ["md_host.cpp", "md_attn.cu", "md_state.cu"]
+SOURCES = ["md_host.cpp", "md_attn.cu", "md_attn_cluster.cu", "md_state.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "--expt-relaxed-constexpr", "-I", INCLUDE]

@@ -39,12 +39,38 @@
 #include <cuda_bf16.h>
 #include <float.h>
 
-#include "md_internal.h"
-#include "md_ptx.cuh"
+#include "md_attn.cuh"
 
 namespace md {
 
 constexpr int NCW_DEFAULT = 4;
+
+/* cuTensorMapEncodeTiled, fetched through the runtime (no link to libcuda) */
+typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+/* The pool viewed as [rows][128] bf16, rows = (layer, page, KV head, K|V,
+ * token); one box = one page's K and V rows x 64 dims, 128-byte swizzled. */
+bool encode_page_map(void *encode, CUtensorMap *m, void *pool, size_t rows, int ps) {
+  const cuuint64_t dims[2] = {(cuuint64_t)D, (cuuint64_t)rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)D * 2};
+  const cuuint32_t box[2] = {64, (cuuint32_t)(2 * ps)}, estr[2] = {1, 1};
+  return ((EncodeTiledFn)encode)(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, pool, dims, strides, box, estr,
+                                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+/* The pool viewed as [(layer, page, KV head)][K|V][token][128]; one box = 16
+ * tokens' K and V rows x 64 dims, so pages of 16 and 32 tokens give the same tile. */
+bool encode_tile_map(void *encode, CUtensorMap *m, void *pool, size_t rows, int ps) {
+  const cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)ps, 2, (cuuint64_t)(rows / (2 * ps))};
+  const cuuint64_t strides[3] = {(cuuint64_t)D * 2, (cuuint64_t)D * 2 * ps, (cuuint64_t)D * 4 * ps};
+  const cuuint32_t box[4] = {64, TILE, 2, 1}, estr[4] = {1, 1, 1, 1};
+  return ((EncodeTiledFn)encode)(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, pool, dims, strides, box, estr,
+                                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 template <int PS, int NCW>
 struct AttnShape {
@@ -97,14 +123,6 @@ __device__ __forceinline__ Unit decode_unit(const AttnParams &p, int u) {
   return un;
 }
 
-/* NEW (a template parameter below): this launch appends the step's new tokens.
- * Free-stack index of sequence b's last page when the step opens it, or -1:
- * the block table holds every page. */
-template <bool NEW>
-__device__ __forceinline__ int tail_pop(const AttnParams &p, int b) {
-  return NEW ? p.nt.tail_pop[b] : -1;
-}
-
 /* Physical ids (and, with region-aligned pages, fills) of pages [from,
  * min(from + 8, to)) of unit x; returns how many.  The loads are
  * independent, so all of them are in flight at once. */
@@ -128,36 +146,6 @@ __device__ __forceinline__ int load_batch(const AttnParams &p, const Unit &x, in
     for (int k = 0; k < 8; ++k) fl[k] = 0;
   }
   return cnt;
-}
-
-__device__ __forceinline__ void raise_status(const AttnParams &p, int code, int diag) {
-  atomicCAS(&p.status[ST_CODE], 0, code);
-  atomicExch(&p.status[ST_DIAG], diag);
-  atomicExch(&p.status[ST_ABORT], 1);
-}
-
-/* Bounded wait on an mbarrier phase; false on abort or timeout. */
-__device__ __noinline__ bool wait_phase(uint32_t bar, uint32_t parity, const AttnParams &p,
-                                        int diag, bool honour_abort) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const long long t0 = globaltimer();
-  while (true) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (honour_abort && ld_volatile(&p.status[ST_ABORT])) return false;
-    if (globaltimer() - t0 > p.spin_limit_ns) {
-      raise_status(p, MD_ERR_DEVICE_TIMEOUT, diag);
-      return false;
-    }
-  }
-}
-
-/* Address of the 16-byte chunk holding (row, d..d+7) of a stage stored as two
- * 64-column halves of 128-byte rows with the TMA 128-byte swizzle. */
-template <int PS>
-__device__ __forceinline__ uint32_t swz(uint32_t stage, int row, int d) {
-  const int half = d >> 6;
-  const int chunk = (d & 63) >> 3;
-  return stage + half * (2 * PS * 128) + row * 128 + ((chunk ^ (row & 7)) << 4);
 }
 
 /* Shared memory of the end-of-unit pass. */
@@ -212,33 +200,16 @@ __device__ __forceinline__ void load_page_ids(const AttnParams &p, const Unit &p
 
 /* One warp puts the new token's K and V rows (row_src: K then V, 256 bytes
  * each, in shared memory; 16 bytes per lane) into the pool and over their
- * stale copy in the stage that holds the sequence's last page, at token
- * `off`; lane 0 of the first layer's KV head 0 starts the token's state. */
+ * stale copy in the stage that holds the sequence's last page, at token `off`. */
 template <int PS>
-__device__ __forceinline__ void append_row(const AttnParams &p, int b, int l, int kvh, int off,
-                                           const uint8_t *row_src, uint8_t *ring, uint32_t ring_u32,
-                                           uint32_t st, int lane) {
-  const int last = p.n_pages[b] - 1;
-  const int pop = tail_pop<true>(p, b);
-  const int phys = pop >= 0 ? p.nt.free_stack[pop] : p.block_table[(size_t)b * p.P_max + last];
+__device__ __forceinline__ void append_row(const AttnParams &p, const Unit &un, int off, const uint8_t *row_src,
+                                           uint8_t *ring, uint32_t ring_u32, uint32_t st, int lane) {
+  const int pop = tail_pop<true>(p, un.b);
+  const int phys =
+      pop >= 0 ? p.nt.free_stack[pop] : p.block_table[(size_t)un.b * p.P_max + p.n_pages[un.b] - 1];
   const uint4 v = *(const uint4 *)(row_src + lane * 16);
-  const int row = (lane < 16 ? 0 : PS) + off;
-  const int d = (lane & 15) * 8;
-  *(uint4 *)(ring + (swz<PS>(st, row, d) - ring_u32)) = v;
-  *(uint4 *)(p.nt.pool + ((((size_t)l * p.P_phys + phys) * p.Hkv + kvh) * 2 * PS + row) * D + d) = v;
-  if (p.nt.init_state && l == p.l0 && kvh == 0 && lane == 0) {
-    const size_t slot = (size_t)phys * PS + off;
-    p.nt.region[slot] = p.nt.tail_region[b];
-    p.nt.t_ref[slot] = p.nt.insert_step;
-    p.nt.t_ins[slot] = p.nt.insert_step;
-    p.nt.a[slot] = 0.f;
-    p.nt.window[slot] = 0.f;
-    p.nt.ahat[slot] = 0.f;
-    p.nt.prio[slot] = 0.f;
-    if (pop >= 0) p.nt.block_table[(size_t)b * p.P_max + last] = phys;
-    p.nt.page_fill[(size_t)b * p.P_max + last] = (uint8_t)(off + 1);
-    p.nt.seq_tokens[b] += 1;
-  }
+  *(uint4 *)(ring + (swz<PS>(st, (lane < 16 ? 0 : PS) + off, (lane & 15) * 8) - ring_u32)) = v;
+  store_new_token(p, un.b, un.l, un.kvh, PS, off, phys, v, lane);
   __syncwarp();
 }
 
@@ -283,10 +254,7 @@ __device__ __forceinline__ void mass_pass(const AttnParams &p, const Unit &pv, i
       const int tk = tk0 + r * NT + tid;
       if (tk >= nvalid) continue;
       if (ALIGNED && (tk % PS) >= f.sfill[tk / PS]) continue;
-      float m = exp2f(s0[r].x - fm[0]) * fz[0] + exp2f(s0[r].y - fm[1]) * fz[1] +
-                exp2f(s0[r].z - fm[2]) * fz[2] + exp2f(s0[r].w - fm[3]) * fz[3];
-      m += exp2f(s1[r].x - fm[4]) * fz[4] + exp2f(s1[r].y - fm[5]) * fz[5] +
-           exp2f(s1[r].z - fm[6]) * fz[6] + exp2f(s1[r].w - fm[7]) * fz[7];
+      const float m = token_mass(s0[r], s1[r], fm, fz);
       const size_t slot_i = (size_t)f.sphys[tk / PS] * PS + (tk % PS);
       if (ROWS)
         mrow[slot_i] = m;
@@ -817,8 +785,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
       const uint32_t st = ring_u32 + s * S::STAGE_BYTES;
       const int fill = ALIGNED ? fillbuf[s] : ntok_seq - (un.p0 + jp) * PS;
       if (NEW && jp == jtail)
-        append_row<PS>(p, un.b, un.l, un.kvh, fill - 1, sQ + (nunit & 1) * S::Q_BYTES + S::NEW_OFF, ring,
-                       ring_u32, st, lane);
+        append_row<PS>(p, un, fill - 1, sQ + (nunit & 1) * S::Q_BYTES + S::NEW_OFF, ring, ring_u32, st, lane);
 
       float acc[S::NT][4];
 #pragma unroll
@@ -1063,11 +1030,6 @@ static __device__ __align__(256) uint8_t g_noalloc_scratch[NOALLOC_BYTES];
 
 namespace {
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
-                                  const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
-                                  const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
 /* What a call needs from its device, found by the first call on that device
  * (with the device current) and kept for the process: the device address of
  * g_noalloc_scratch and the attention CTAs resident at once, for pages of 16
@@ -1079,9 +1041,9 @@ struct NoallocDevice {
 constexpr int NOALLOC_MAX_DEVICES = 128;
 std::mutex g_noalloc_mu;
 NoallocDevice g_noalloc_dev[NOALLOC_MAX_DEVICES];
-EncodeTiledFn g_encode = nullptr;
+void *g_encode = nullptr;   // the driver's tensor-map encoder
 
-cudaError_t noalloc_device(int ps, void **base, int *grid_limit, EncodeTiledFn *encode) {
+cudaError_t noalloc_device(int ps, void **base, int *grid_limit, void **encode) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -1096,6 +1058,7 @@ cudaError_t noalloc_device(int ps, void **base, int *grid_limit, EncodeTiledFn *
   }
   int &gl = d.grid_limit[ps == 32 ? 1 : 0];
   if (gl <= 0) {
+    if (md::cluster_prepare() != cudaSuccess) return cudaErrorUnknown;
     gl = md::attention_grid_limit(ps);
     if (gl <= 0) return cudaErrorUnknown;
   }
@@ -1105,7 +1068,7 @@ cudaError_t noalloc_device(int ps, void **base, int *grid_limit, EncodeTiledFn *
     e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
     if (e != cudaSuccess) return e;
     if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorUnknown;
-    g_encode = (EncodeTiledFn)fn;
+    g_encode = fn;
   }
   *base = d.base;
   *grid_limit = gl;
@@ -1178,7 +1141,7 @@ extern "C" __attribute__((visibility("default"))) md_status md_attend_mass_noall
 
   void *base = nullptr;
   int grid_limit = 0;
-  EncodeTiledFn encode = nullptr;
+  void *encode = nullptr;
   if (noalloc_device(ps, &base, &grid_limit, &encode) != cudaSuccess) return MD_ERR_CUDA;
 
   AttnParams ap;
@@ -1251,19 +1214,19 @@ extern "C" __attribute__((visibility("default"))) md_status md_attend_mass_noall
   ap.extra_arrivals = 0;
 
   CUtensorMap tmap;
-  cuuint64_t dims[2] = {(cuuint64_t)D, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)D * 2};
-  cuuint32_t box[2] = {64, (cuuint32_t)(2 * ps)};
-  cuuint32_t estr[2] = {1, 1};
-  if (encode(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void *)kv_pool_dev, dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return MD_ERR_INVALID_ARG;
+  cudaStream_t st = (cudaStream_t)stream;
+  cudaError_t e;
+  const ClusterPlan plan = cluster_plan(ap);
+  if (plan.C > 0) {   // needs no scratch: nothing of the array is touched
+    if (!encode_tile_map(encode, &tmap, (void *)kv_pool_dev, rows, ps)) return MD_ERR_INVALID_ARG;
+    e = launch_cluster(ap, plan, false, tmap, st);
+    return e == cudaSuccess ? MD_OK : MD_ERR_CUDA;
+  }
+  if (!encode_page_map(encode, &tmap, (void *)kv_pool_dev, rows, ps)) return MD_ERR_INVALID_ARG;
 
   /* the array keeps the previous call's contents: counters and status words
    * must start at zero */
-  cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e = cudaMemsetAsync(s8, 0, NOALLOC_STATUS_BYTES + best.counters_bytes, st);
+  e = cudaMemsetAsync(s8, 0, NOALLOC_STATUS_BYTES + best.counters_bytes, st);
   if (e != cudaSuccess) return MD_ERR_CUDA;
   e = launch_attention(ap, tmap, best.grid, st);
   return e == cudaSuccess ? MD_OK : MD_ERR_CUDA;

@@ -51,7 +51,7 @@ struct md_ctx {
   Layout lay;
   uint8_t *ws = nullptr;
   cudaStream_t stream = nullptr;
-  CUtensorMap tmap;
+  CUtensorMap tmap, tmap_tile;   // boxes of the persistent and of the cluster kernel
   int grid_limit = 0;
   RegionTable reg;
   HostMirror m;
@@ -449,13 +449,10 @@ void plan_attention(md_ctx *c, int batch, int layers, AttnParams &ap, int *grid)
     if (P > 0) ch = std::min(std::min((P + bestT - 1) / bestT, cmax), P);
     ap.chunks[b] = ch;
     ap.unit_start[b] = (int)U;
-    ap.n_pages[b] = P;
-    ap.n_tokens[b] = (int)c->n_tokens[b];
     U += (long long)items * ch;
   }
   ap.unit_start[batch] = (int)U;
   ap.total_units = (int)U;
-  ap.n_seqs = batch;
   ap.units_per_seq = batch > 0 ? (int)(U / batch) : 0;
   for (int b = 0; b < batch && ap.units_per_seq > 0; ++b)
     if (ap.unit_start[b + 1] - ap.unit_start[b] != ap.units_per_seq) ap.units_per_seq = 0;
@@ -555,6 +552,7 @@ MD_API md_status md_create(const md_config *cfg, md_ctx **out) {
   c->m.free_top = cfg->num_phys_pages;
 
   cudaError_t e = attention_prepare(cfg->page_size);
+  if (e == cudaSuccess) e = cluster_prepare();
   if (e != cudaSuccess) {
     delete c;
     return MD_ERR_CUDA;
@@ -575,9 +573,6 @@ MD_API md_status md_create(const md_config *cfg, md_ctx **out) {
     delete c;
     return MD_ERR_CAPACITY;
   }
-  /* TMA descriptor over the pool viewed as [rows][128] bf16, rows = (layer,
-   * page, KV head, K|V, token); one box = one page's K and V rows x 64 dims,
-   * 128-byte swizzled. */
   void *fn = nullptr;
   cudaDriverEntryPointQueryResult q;
   e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
@@ -585,21 +580,9 @@ MD_API md_status md_create(const md_config *cfg, md_ctx **out) {
     delete c;
     return MD_ERR_CUDA;
   }
-  typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
-                               const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
-                               const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  const cuuint64_t rows = (cuuint64_t)cfg->num_layers * cfg->num_phys_pages *
-                          cfg->num_kv_heads * 2 * cfg->page_size;
-  cuuint64_t dims[2] = {(cuuint64_t)D, rows};
-  cuuint64_t strides[1] = {(cuuint64_t)D * 2};
-  cuuint32_t box[2] = {64, (cuuint32_t)(2 * cfg->page_size)};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult cr = ((EncodeFn)fn)(&c->tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, c->ws + lay.pool,
-                               dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (cr != CUDA_SUCCESS) {
+  const size_t rows = (size_t)cfg->num_layers * cfg->num_phys_pages * cfg->num_kv_heads * 2 * cfg->page_size;
+  if (!encode_page_map(fn, &c->tmap, c->ws + lay.pool, rows, cfg->page_size) ||
+      !encode_tile_map(fn, &c->tmap_tile, c->ws + lay.pool, rows, cfg->page_size)) {
     delete c;
     return MD_ERR_CUDA;
   }
@@ -828,36 +811,34 @@ md_status append_step(md_ctx *c, int batch, const void *k_new, const void *v_new
 md_status run_attention(md_ctx *c, int batch, int l0, int L, int q_layers, const void *q_dev,
                         const void *k_new, const void *v_new, void *out_dev) {
   const md_config &cf = c->cfg;
-  AttnParams atp;
-  memset(&atp, 0, sizeof(atp));
-  atp.q = (const uint16_t *)q_dev;
-  atp.out = (uint16_t *)out_dev;
-  atp.block_table = ptr<int32_t>(c, c->lay.block_table);
-  atp.page_fill = cf.region_aligned_pages ? ptr<uint8_t>(c, c->lay.page_fill) : nullptr;
-  atp.mass_acc = ptr<unsigned long long>(c, c->lay.mass_acc);
-  atp.scratch = ptr<float>(c, c->lay.scratch);
-  atp.partials = ptr<float>(c, c->lay.partials);
-  atp.counters = ptr<int>(c, c->lay.counters);
-  atp.status = ptr<int>(c, c->lay.status);
-  atp.L = cf.num_layers;
-  atp.l0 = l0;
-  atp.L_launch = L;
-  atp.q_layers = q_layers;
-  atp.Hq = cf.num_q_heads;
-  atp.Hkv = cf.num_kv_heads;
-  atp.G = cf.num_q_heads / cf.num_kv_heads;
-  atp.ps = cf.page_size;
-  atp.P_phys = cf.num_phys_pages;
-  atp.P_max = cf.max_pages_per_seq;
-  atp.slots = (long long)c->lay.slots;
-  atp.scratch_tokens = c->lay.scratch_tokens;
-  atp.chunk_stride = c->lay.chunk_stride;
-  atp.scale_log2 = (float)(1.4426950408889634 / sqrt((double)D));
-  atp.spin_limit_ns = c->spin_limit_ns;
-  atp.extra_arrivals = c->extra_arrivals;
-  c->extra_arrivals = 0;
+  AttnBase base;
+  memset(&base, 0, sizeof(base));
+  base.q = (const uint16_t *)q_dev;
+  base.out = (uint16_t *)out_dev;
+  base.block_table = ptr<int32_t>(c, c->lay.block_table);
+  base.page_fill = cf.region_aligned_pages ? ptr<uint8_t>(c, c->lay.page_fill) : nullptr;
+  base.mass_acc = ptr<unsigned long long>(c, c->lay.mass_acc);
+  base.status = ptr<int>(c, c->lay.status);
+  base.L = cf.num_layers;
+  base.l0 = l0;
+  base.L_launch = L;
+  base.q_layers = q_layers;
+  base.Hq = cf.num_q_heads;
+  base.Hkv = cf.num_kv_heads;
+  base.G = cf.num_q_heads / cf.num_kv_heads;
+  base.ps = cf.page_size;
+  base.P_phys = cf.num_phys_pages;
+  base.P_max = cf.max_pages_per_seq;
+  base.slots = (long long)c->lay.slots;
+  base.scale_log2 = (float)(1.4426950408889634 / sqrt((double)D));
+  base.spin_limit_ns = c->spin_limit_ns;
+  base.n_seqs = batch;
+  for (int b = 0; b < batch; ++b) {
+    base.n_tokens[b] = (int)c->n_tokens[b];
+    base.n_pages[b] = c->n_pages[b];
+  }
   if (k_new) {
-    NewTokens &nt = atp.nt;
+    NewTokens &nt = base.nt;
     nt.k_new = (const uint16_t *)k_new;
     nt.v_new = (const uint16_t *)v_new;
     nt.sb = (long long)L * cf.num_kv_heads * D;
@@ -882,11 +863,31 @@ md_status run_attention(md_ctx *c, int batch, int l0, int L, int q_layers, const
       nt.tail_region[b] = (uint8_t)c->tail_region[b];
     }
   }
+  /* the debug knobs of the persistent kernel's planner and exchange keep that kernel */
+  const bool knobs = c->grid_cap > 0 || c->force_chunks > 0 || c->extra_arrivals > 0;
+  const ClusterPlan plan = knobs ? ClusterPlan{} : cluster_plan(base);
+  cudaEvent_t e0;
+  cudaError_t e;
+  if (plan.C > 0) {
+    prof_begin(c, &e0);
+    e = launch_cluster(base, plan, k_new && l0 > 0, c->tmap_tile, c->stream);
+    prof_end(c, STAGE_ATTN, e0);
+    return e == cudaSuccess ? MD_OK : cuda_fail(c, e, "attention launch");
+  }
+  AttnParams atp;
+  memset(&atp, 0, sizeof(atp));
+  (AttnBase &)atp = base;
+  atp.scratch = ptr<float>(c, c->lay.scratch);
+  atp.partials = ptr<float>(c, c->lay.partials);
+  atp.counters = ptr<int>(c, c->lay.counters);
+  atp.scratch_tokens = c->lay.scratch_tokens;
+  atp.chunk_stride = c->lay.chunk_stride;
+  atp.extra_arrivals = c->extra_arrivals;
+  c->extra_arrivals = 0;
   int grid = 1;
   plan_attention(c, batch, L, atp, &grid);
-  cudaEvent_t e0;
   prof_begin(c, &e0);
-  cudaError_t e = launch_attention(atp, c->tmap, grid, c->stream);
+  e = launch_attention(atp, c->tmap, grid, c->stream);
   prof_end(c, STAGE_ATTN, e0);
   if (e != cudaSuccess) return cuda_fail(c, e, "attention launch");
   return MD_OK;

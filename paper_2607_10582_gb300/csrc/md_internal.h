@@ -100,7 +100,8 @@ struct NewTokens {
   uint8_t tail_region[MD_MAX_BATCH];
 };
 
-struct AttnParams {
+/* What both attention kernels take. */
+struct AttnBase {
   const uint16_t *q;
   uint16_t *out;
   const int32_t *block_table;
@@ -108,27 +109,55 @@ struct AttnParams {
                              // full up to n_tokens
   unsigned long long *mass_acc;   // [slots] fixed-point mass of the step, or null:
   float *mass;                    // [L*Hkv][slots] one fp32 row per (layer, KV head)
-  float *scratch;      // [grid][2][scratch_tokens][8]
-  float *partials;     // [items][chunk_stride][PARTIAL_FLOATS]
-  int *counters;       // [items]
   int *status;         // sticky device status words
   int L, Hq, Hkv, G, ps, P_phys, P_max;   // L: layers of the model
   int l0, L_launch;    // layers [l0, l0 + L_launch) attended by this launch
   int q_layers;        // layers held by the q / out tensors (L or 1)
   long long slots;
-  int scratch_tokens;  // scratch row capacity per CTA slot (tokens)
-  int chunk_stride;    // partial slots reserved per item
   float scale_log2;    // log2(e) / sqrt(D)
   long long spin_limit_ns;
-  int extra_arrivals;
-  NewTokens nt;
-  int n_seqs, total_units;
-  int units_per_seq;   // > 0: every sequence has this many units (no search)
+  int n_seqs;
   int n_tokens[MD_MAX_BATCH];
   int n_pages[MD_MAX_BATCH];
+  NewTokens nt;
+};
+
+/* The persistent kernel (md_attn.cu). */
+struct AttnParams : AttnBase {
+  float *scratch;      // [grid][2][scratch_tokens][8]
+  float *partials;     // [items][chunk_stride][PARTIAL_FLOATS]
+  int *counters;       // [items]
+  int scratch_tokens;  // scratch row capacity per CTA slot (tokens)
+  int chunk_stride;    // partial slots reserved per item
+  int extra_arrivals;
+  int total_units;
+  int units_per_seq;   // > 0: every sequence has this many units (no search)
   int chunks[MD_MAX_BATCH];
   int unit_start[MD_MAX_BATCH + 1];
 };
+
+/* The cluster kernel (md_attn_cluster.cu): a cluster of C CTAs of 4 or 8
+ * warps per (sequence, layer, KV head), each warp with up to 32 tiles of TILE
+ * tokens. */
+constexpr int TILE = 16;
+constexpr int MAX_CLUSTER = 16;
+struct ClusterParams : AttnBase {
+  int C;               // CTAs per item
+  int warp_tiles;      // most tiles of any warp (sizes the score rows)
+  int early;           // K/V copies may start before the kernel ahead has finished
+  int out16;           // out is 16-byte aligned
+};
+struct ClusterPlan {
+  int C = 0;           // CTAs per item, or 0: the persistent kernel
+  int warps = 4, warp_tiles = 0;
+};
+cudaError_t cluster_prepare();
+ClusterPlan cluster_plan(const AttnBase &p);
+cudaError_t launch_cluster(const AttnBase &p, const ClusterPlan &plan, bool early, const CUtensorMap &tmap,
+                           cudaStream_t s);
+/* The tensor maps of the K/V pool (encode: the driver's cuTensorMapEncodeTiled). */
+bool encode_page_map(void *encode, CUtensorMap *m, void *pool, size_t rows, int ps);
+bool encode_tile_map(void *encode, CUtensorMap *m, void *pool, size_t rows, int ps);
 cudaError_t launch_attention(const AttnParams &p, const CUtensorMap &tmap, int grid,
                              cudaStream_t s);
 int attention_grid_limit(int ps);     // CTAs resident at once (0 on error)

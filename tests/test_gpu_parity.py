@@ -407,6 +407,46 @@ def test_entry_points_mixed_step_by_step():
     ls.check_layout()
 
 
+@pytest.mark.parametrize("L,Hq,Hkv,ps,lengths,aligned", [
+    (1, 8, 1, 16, [15], 0),                                  # one tile, one CTA
+    (1, 3, 1, 16, [431], 0),                                 # clusters of 8, G = 3 padded heads
+    (1, 16, 2, 32, [1, 17, 4095], 0),                        # clusters of 16: most chunks of the short ones are empty
+    (2, 28, 4, 32, [1000] * 3 + [33], 1),                    # region-aligned pages, half-empty second tiles
+    (1, 12, 2, 16, [1500 + 16 * i for i in range(12)], 0),   # clusters of CTAs of 8 warps
+    (2, 16, 2, 16, [300 + 7 * i for i in range(40)], 0),     # one CTA per item, more than one wave
+    (3, 5, 1, 16, [1790 - 25 * i for i in range(60)], 0),    # the same with 8 warps
+])
+def test_cluster_attention_follows_the_oracle(L, Hq, Hkv, ps, lengths, aligned):
+    """Launch shapes that take the cluster attention kernel in each of its
+    forms, with sizes at the edges of tiles, warps and chunks."""
+    w = synth.custom_workload("cluster", L=L, Hq=Hq, Hkv=Hkv, page_size=ps, lengths=lengths, budget_frac=0.7,
+                              steps=3, seed=41, structured=True)
+    w.extra["region_aligned"] = bool(aligned)
+    ls = Lockstep(w).run()
+    ls.check_layout()
+
+
+@pytest.mark.parametrize("n", [40, 900])
+def test_output_at_any_address(n):
+    """The output may start at any 2-byte address: the wide stores are taken
+    only where it is aligned for them."""
+    w = synth.custom_workload("addr", L=1, Hq=16, Hkv=2, page_size=16, lengths=[n], budget_frac=1.0, steps=1, seed=43)
+    outs = []
+    for shift in (0, 1, 4):
+        c = md.Cache(1, 16, 2, 16, 1, 80, 80)
+        k, v = synth.kv_host(w.seed, 0, 1, 2, 0, n, w.regions[0])
+        c.append_tokens(0, w.regions[0], to_dev(k), to_dev(v))
+        kn, vn = synth.step_kv_host(w.seed, [n], [6], 1, 2)
+        buf = torch.zeros(16 * 128 + 8, dtype=torch.int16, device="cuda")
+        c.decode_step(1, to_dev(synth.q_host(w.seed, 1, 1, 16, 2, 1)), to_dev(kn), to_dev(vn), [6],
+                      buf.data_ptr() + 2 * shift)
+        assert c.sync() == md.MD_OK
+        assert int(buf[:shift].abs().sum()) == 0 and int(buf[shift + 16 * 128:].abs().sum()) == 0
+        outs.append(buf[shift:shift + 16 * 128].clone())
+        c.close()
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+
+
 @pytest.mark.parametrize("ps,aligned", [(16, 0), (32, 0), (16, 1), (32, 1)])
 @pytest.mark.parametrize("entry", ["device", "layers"])
 def test_append_inside_attention_writes_what_the_append_kernel_writes(ps, aligned, entry):
