@@ -202,6 +202,17 @@ void mirror_token(md_ctx *c, int b, int r) {
   c->n_tokens[b] += 1;
 }
 
+/* The same for m consecutive tokens of region r. */
+void mirror_run(md_ctx *c, int b, int r, int m) {
+  while (m > 0) {
+    mirror_token(c, b, r);
+    const int more = std::min(m - 1, c->cfg.page_size - c->tail_fill[b]);   // the rest fits the page
+    c->tail_fill[b] += more;
+    c->n_tokens[b] += more;
+    m -= 1 + more;
+  }
+}
+
 int64_t cached_tokens(const md_ctx *c) {
   int64_t s = 0;
   for (auto v : c->n_pages) s += v;
@@ -614,6 +625,31 @@ MD_API md_status md_set_region_params(md_ctx *c, int region, float base, float h
   return MD_OK;
 }
 
+namespace {
+AppendTo append_to(md_ctx *c) {
+  const md_config &cf = c->cfg;
+  AppendTo d;
+  d.pool = ptr<uint16_t>(c, c->lay.pool);
+  d.block_table = ptr<int32_t>(c, c->lay.block_table);
+  d.free_stack = ptr<int32_t>(c, c->lay.free_stack);
+  d.region = ptr<uint8_t>(c, c->lay.region);
+  d.a = ptr<float>(c, c->lay.a);
+  d.window = ptr<float>(c, c->lay.window);
+  d.ahat = ptr<float>(c, c->lay.ahat);
+  d.prio = ptr<float>(c, c->lay.prio);
+  d.t_ref = ptr<int32_t>(c, c->lay.t_ref);
+  d.t_ins = ptr<int32_t>(c, c->lay.t_ins);
+  d.page_fill = ptr<uint8_t>(c, c->lay.page_fill);
+  d.seq_tokens = ptr<int32_t>(c, c->lay.seq_tokens);
+  d.L = cf.num_layers;
+  d.Hkv = cf.num_kv_heads;
+  d.ps = cf.page_size;
+  d.P_phys = cf.num_phys_pages;
+  d.P_max = cf.max_pages_per_seq;
+  return d;
+}
+}  // namespace
+
 MD_API md_status md_append_tokens(md_ctx *c, int seq, int n, const uint8_t *regions_host,
                                   const int32_t *steps_host, const void *k_dev,
                                   const void *v_dev) {
@@ -631,22 +667,31 @@ MD_API md_status md_append_tokens(md_ctx *c, int seq, int n, const uint8_t *regi
     for (int i = 0; i < n; ++i)
       if (steps_host[i] > c->m.t) return fail(c, MD_ERR_INVALID_ARG, "insertion step in the future");
   const int ps = cf.page_size;
-  /* where the tokens go: the same page-opening rule as the mirror */
-  std::vector<int32_t> slots(n);
+  /* The tokens as runs of one region, insertion step and consecutive slots,
+   * placed by the mirror's page-opening rule. */
+  AppendTokensParams ap;
+  int n_runs = 0;
   long long pages_after = c->n_pages[seq];
   {
     int fill = c->tail_fill[seq], treg = c->tail_region[seq];
-    for (int i = 0; i < n; ++i) {
-      const int r = regions_host[i];
+    for (int i = 0; i < n;) {
+      const int r = regions_host[i], step = steps_host ? steps_host[i] : (int)c->m.t;
+      int m = 1;
+      while (i + m < n && regions_host[i + m] == r && (!steps_host || steps_host[i + m] == step)) ++m;
       if (pages_after == 0 || fill == ps || (cf.region_aligned_pages && treg != r)) {
         ++pages_after;
         fill = 0;
       }
-      slots[i] = (int32_t)((pages_after - 1) * ps + fill);
-      ++fill;
+      if (n_runs < MAX_RUNS) ap.runs[n_runs] = {i, (int)((pages_after - 1) * ps + fill), step, r};
+      ++n_runs;
+      const int over = std::max(0, m - (ps - fill));   // tokens past the page being filled
+      pages_after += (over + ps - 1) / ps;
+      fill = over > 0 ? over - (over + ps - 1) / ps * ps + ps : fill + m;
       treg = r;
+      i += m;
     }
   }
+  const bool by_runs = n_runs <= MAX_RUNS;
   const long long new_pages = pages_after - c->n_pages[seq];
   if (pages_after > cf.max_pages_per_seq)
     return fail(c, MD_ERR_CAPACITY, "sequence %d would need %lld pages (max %d)", seq,
@@ -658,56 +703,50 @@ MD_API md_status md_append_tokens(md_ctx *c, int seq, int n, const uint8_t *regi
     md_status st = launch_fold(c);
     if (st != MD_OK) return st;
   }
-  cudaError_t e = cudaMemcpyAsync(c->ws + c->lay.staging_regions, regions_host, (size_t)n,
-                                  cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess && steps_host)
-    e = cudaMemcpyAsync(c->ws + c->lay.staging_steps, steps_host, (size_t)n * 4,
-                        cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess && cf.region_aligned_pages)
-    e = cudaMemcpyAsync(c->ws + c->lay.staging_slots, slots.data(), (size_t)n * 4,
-                        cudaMemcpyHostToDevice, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "staging copy");
-  AppendParams ap;
-  memset(&ap, 0, sizeof(ap));
-  ap.pool = ptr<uint16_t>(c, c->lay.pool);
-  ap.block_table = ptr<int32_t>(c, c->lay.block_table);
-  ap.free_stack = ptr<int32_t>(c, c->lay.free_stack);
-  ap.region = ptr<uint8_t>(c, c->lay.region);
-  ap.a = ptr<float>(c, c->lay.a);
-  ap.window = ptr<float>(c, c->lay.window);
-  ap.ahat = ptr<float>(c, c->lay.ahat);
-  ap.prio = ptr<float>(c, c->lay.prio);
-  ap.t_ref = ptr<int32_t>(c, c->lay.t_ref);
-  ap.t_ins = ptr<int32_t>(c, c->lay.t_ins);
-  ap.page_fill = ptr<uint8_t>(c, c->lay.page_fill);
-  ap.seq_tokens = ptr<int32_t>(c, c->lay.seq_tokens);
-  ap.slots_dev = cf.region_aligned_pages ? ptr<int32_t>(c, c->lay.staging_slots) : nullptr;
+  cudaError_t e = cudaSuccess;
+  if (!by_runs) {
+    e = cudaMemcpyAsync(c->ws + c->lay.staging_regions, regions_host, (size_t)n, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess && steps_host)
+      e = cudaMemcpyAsync(c->ws + c->lay.staging_steps, steps_host, (size_t)n * 4, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess && cf.region_aligned_pages) {
+      std::vector<int32_t> slots(n);
+      int fill = c->tail_fill[seq], treg = c->tail_region[seq], pages = c->n_pages[seq];
+      for (int i = 0; i < n; ++i) {
+        if (pages == 0 || fill == ps || treg != regions_host[i]) {
+          ++pages;
+          fill = 0;
+        }
+        slots[i] = (pages - 1) * ps + fill++;
+        treg = regions_host[i];
+      }
+      e = cudaMemcpyAsync(c->ws + c->lay.staging_slots, slots.data(), (size_t)n * 4, cudaMemcpyHostToDevice, c->stream);
+    }
+    if (e != cudaSuccess) return cuda_fail(c, e, "staging copy");
+  }
+  ap.to = append_to(c);
   ap.k_src = (const uint16_t *)k_dev;
   ap.v_src = (const uint16_t *)v_dev;
-  ap.sb = 0;
-  ap.sl = (long long)cf.num_kv_heads * n * D;
-  ap.sh = (long long)n * D;
-  ap.si = D;
-  ap.regions_dev = ptr<uint8_t>(c, c->lay.staging_regions);
-  ap.steps_dev = steps_host ? ptr<int32_t>(c, c->lay.staging_steps) : nullptr;
-  ap.L = cf.num_layers;
-  ap.Hkv = cf.num_kv_heads;
-  ap.ps = ps;
-  ap.P_phys = cf.num_phys_pages;
-  ap.P_max = cf.max_pages_per_seq;
-  ap.n_seqs = 1;
-  ap.n_per_seq = n;
-  ap.seq0 = seq;
+  ap.regions_dev = by_runs ? nullptr : ptr<uint8_t>(c, c->lay.staging_regions);
+  ap.steps_dev = !by_runs && steps_host ? ptr<int32_t>(c, c->lay.staging_steps) : nullptr;
+  ap.slots_dev = !by_runs && cf.region_aligned_pages ? ptr<int32_t>(c, c->lay.staging_slots) : nullptr;
+  ap.seq = seq;
+  ap.n = n;
+  ap.tok0 = ap.runs[0].slot;
   ap.insert_step = (int)c->m.t;
-  ap.tok0[0] = slots[0];
-  ap.pages_before[0] = c->n_pages[seq];
-  ap.pop_base[0] = (int)(c->m.free_top - 1);
+  ap.pages_before = c->n_pages[seq];
+  ap.pop_base = (int)(c->m.free_top - 1);
+  ap.n_runs = std::min(n_runs, MAX_RUNS);
   cudaEvent_t e0;
   prof_begin(c, &e0);
-  e = launch_append(ap, c->stream);
+  e = launch_append_tokens(ap, cf.region_aligned_pages != 0, c->stream);
   prof_end(c, STAGE_APPEND, e0);
   if (e != cudaSuccess) return cuda_fail(c, e, "append launch");
-  for (int i = 0; i < n; ++i) mirror_token(c, seq, regions_host[i]);
+  for (int i = 0; i < n;) {
+    int m = 1;
+    while (i + m < n && regions_host[i + m] == regions_host[i]) ++m;
+    mirror_run(c, seq, regions_host[i], m);
+    i += m;
+  }
   c->m.free_top -= new_pages;
   return MD_OK;
 }
@@ -735,29 +774,6 @@ md_status check_step(md_ctx *c, int batch, const uint8_t *new_region_host) {
   return MD_OK;
 }
 
-void fill_append_common(md_ctx *c, AppendParams &ap) {
-  const md_config &cf = c->cfg;
-  memset(&ap, 0, sizeof(ap));
-  ap.pool = ptr<uint16_t>(c, c->lay.pool);
-  ap.block_table = ptr<int32_t>(c, c->lay.block_table);
-  ap.free_stack = ptr<int32_t>(c, c->lay.free_stack);
-  ap.region = ptr<uint8_t>(c, c->lay.region);
-  ap.a = ptr<float>(c, c->lay.a);
-  ap.window = ptr<float>(c, c->lay.window);
-  ap.ahat = ptr<float>(c, c->lay.ahat);
-  ap.prio = ptr<float>(c, c->lay.prio);
-  ap.t_ref = ptr<int32_t>(c, c->lay.t_ref);
-  ap.t_ins = ptr<int32_t>(c, c->lay.t_ins);
-  ap.page_fill = ptr<uint8_t>(c, c->lay.page_fill);
-  ap.seq_tokens = ptr<int32_t>(c, c->lay.seq_tokens);
-  ap.Hkv = cf.num_kv_heads;
-  ap.ps = cf.page_size;
-  ap.P_phys = cf.num_phys_pages;
-  ap.P_max = cf.max_pages_per_seq;
-  ap.n_per_seq = 1;
-  ap.seq0 = 0;
-}
-
 /* Start of a decode step: fold the step before it, advance t, take the new
  * tokens' pages.  The append launch or the attention launch then writes the
  * rows and the tokens' state. */
@@ -781,27 +797,20 @@ md_status begin_step(md_ctx *c, int batch, const uint8_t *new_region_host) {
  * attention units' reads of two short rows each would pay its latency. */
 md_status append_step(md_ctx *c, int batch, const void *k_new, const void *v_new) {
   const md_config &cf = c->cfg;
-  AppendParams ap;
-  fill_append_common(c, ap);
+  AppendStepParams ap;
+  ap.to = append_to(c);
   ap.k_src = (const uint16_t *)k_new;
   ap.v_src = (const uint16_t *)v_new;
-  ap.sb = (long long)cf.num_layers * cf.num_kv_heads * D;
-  ap.sl = (long long)cf.num_kv_heads * D;
-  ap.sh = D;
-  ap.si = 0;
-  ap.L = cf.num_layers;
   ap.n_seqs = batch;
   ap.insert_step = (int)c->m.t;
   for (int b = 0; b < batch; ++b) {
-    const bool opened = c->tail_pop[b] >= 0;
     ap.tok0[b] = (c->n_pages[b] - 1) * cf.page_size + c->tail_fill[b] - 1;
-    ap.pages_before[b] = c->n_pages[b] - (opened ? 1 : 0);
-    ap.pop_base[b] = c->tail_pop[b];
-    ap.regions_param[b] = (uint8_t)c->tail_region[b];
+    ap.pop[b] = c->tail_pop[b];
+    ap.regions[b] = (uint8_t)c->tail_region[b];
   }
   cudaEvent_t e0;
   prof_begin(c, &e0);
-  cudaError_t e = launch_append(ap, c->stream);
+  cudaError_t e = launch_append_step(ap, c->stream);
   prof_end(c, STAGE_APPEND, e0);
   return e == cudaSuccess ? MD_OK : cuda_fail(c, e, "append launch");
 }

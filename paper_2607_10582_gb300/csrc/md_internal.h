@@ -50,28 +50,53 @@ struct Layout {
 size_t compute_layout(const md_config &c, Layout *lay);
 
 /* ------------------------------------------------------------- append --- */
-struct AppendParams {
+/* The arrays an append writes. */
+struct AppendTo {
   uint16_t *pool;
   int32_t *block_table;
   const int32_t *free_stack;
   uint8_t *region;
   float *a, *window, *ahat, *prio;
   int32_t *t_ref, *t_ins;
-  const uint16_t *k_src, *v_src;
-  long long sb, sl, sh, si;              // element strides of the source (seq, layer, head, token)
-  const uint8_t *regions_dev;            // per token (prefill) or null
-  const int32_t *steps_dev;              // per token (prefill) or null
-  const int32_t *slots_dev;              // per token slot in the sequence (prefill) or null
   uint8_t *page_fill;                    // [max_batch][P_max] tokens per page
   int32_t *seq_tokens;                   // [max_batch] tokens per sequence
   int L, Hkv, ps, P_phys, P_max;
-  int n_seqs, n_per_seq, seq0, insert_step;
-  int tok0[MD_MAX_BATCH];                // slot of the first token (slots_dev == null)
-  int pages_before[MD_MAX_BATCH];        // pages of the sequence before this append
-  int pop_base[MD_MAX_BATCH];            // free-stack index of the first page taken
-  uint8_t regions_param[MD_MAX_BATCH];   // decode: region of each new token
 };
-cudaError_t launch_append(const AppendParams &p, cudaStream_t s);
+/* One new token for each of n_seqs sequences (a decode step's append as a
+ * launch of its own); k_src, v_src are [n_seqs][L][Hkv][D]. */
+struct AppendStepParams {
+  AppendTo to;
+  const uint16_t *k_src, *v_src;
+  int n_seqs, insert_step;
+  int tok0[MD_MAX_BATCH];                // slot of the token in its sequence
+  int pop[MD_MAX_BATCH];                 // free-stack index of the page it opens, or -1
+  uint8_t regions[MD_MAX_BATCH];
+};
+cudaError_t launch_append_step(const AppendStepParams &p, cudaStream_t s);
+
+/* n tokens for one sequence (a prompt, a tool's output); k_src, v_src are
+ * [L][Hkv][n][D].  The tokens' labels, insertion steps and slots come as runs
+ * in the launch parameters; a text of more runs than fit goes through arrays
+ * in the workspace instead (regions_dev, and where needed the others). */
+constexpr int MAX_RUNS = 512;
+struct AppendRun {
+  int start;                             // first token of the run
+  int slot;                              // its slot in the sequence (then consecutive)
+  int step, region;
+};
+struct AppendTokensParams {
+  AppendTo to;
+  const uint16_t *k_src, *v_src;
+  const uint8_t *regions_dev;            // per token, or null: runs
+  const int32_t *steps_dev;              // per token, or null: insert_step
+  const int32_t *slots_dev;              // per token, or null: consecutive from tok0
+  int seq, n, tok0, insert_step;
+  int pages_before;                      // pages of the sequence before this append
+  int pop_base;                          // free-stack index of the first page taken
+  int n_runs;
+  AppendRun runs[MAX_RUNS];
+};
+cudaError_t launch_append_tokens(const AppendTokensParams &p, bool aligned, cudaStream_t s);
 
 /* ---------------------------------------------------------- attention --- */
 /* The decode step's new tokens, one per sequence, when the attention launch

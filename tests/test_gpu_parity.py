@@ -448,6 +448,47 @@ def test_output_at_any_address(n):
 
 
 @pytest.mark.parametrize("ps,aligned", [(16, 0), (32, 0), (16, 1), (32, 1)])
+@pytest.mark.parametrize("runs", ["spans", "single tokens"])
+def test_append_in_one_call_and_in_pieces(ps, aligned, runs):
+    """The same tokens appended in one call and in pieces of odd sizes leave
+    the same pool, token state and page tables, bit for bit, with few runs of
+    equal labels and steps (passed in the launch parameters) and with more than
+    fit there (passed through the workspace)."""
+    L, Hkv, n = 2, 3, 1333
+    rng = np.random.default_rng(11)
+    lab = np.repeat(rng.integers(0, 7, 40), 34)[:n].astype(np.uint8) if runs == "spans" else \
+        (np.arange(n) * 5 % 7).astype(np.uint8)
+    step = -(np.arange(n, dtype=np.int32)[::-1] // 100) if runs == "spans" else -np.arange(n, dtype=np.int32) % 50 - 49
+    k, v = synth.kv_host(13, 0, L, Hkv, 0, n, lab)
+    kd, vd = to_dev(k), to_dev(v)
+    states = []
+    for sizes in ([n], [1, 15, 16, 17, 31, 33, 5, 700, 64, n]):
+        c = md.Cache(L, 6, Hkv, ps, 2, n, n + 4, region_aligned_pages=aligned)
+        c.set_region_params(0, 1.0, 10.0, True)
+        i = 0
+        for m in sizes:
+            m = min(m, n - i)
+            c.append_tokens(1, lab[i:i + m], kd[:, :, i:i + m].contiguous(), vd[:, :, i:i + m].contiguous(), step[i:i + m])
+            i += m
+        assert c.query(md.MD_QUERY_TOKENS, 1) == n
+        states.append([c.get_state(w) for w in (
+            md.MD_STATE_POOL, md.MD_STATE_REGION, md.MD_STATE_T_INS, md.MD_STATE_T_REF, md.MD_STATE_A,
+            md.MD_STATE_BLOCK_TABLE, md.MD_STATE_PAGE_FILL, md.MD_STATE_SEQ_TOKENS)] +
+            [torch.tensor([c.query(q, 1) for q in (md.MD_QUERY_PAGES, md.MD_QUERY_PINNED_PAGES, md.MD_QUERY_FREE_TOP)])])
+        slots = c.get_state(md.MD_STATE_BLOCK_TABLE)[1].cpu().numpy()
+        if not aligned:      # and the pool holds the tokens where the table says
+            at = torch.from_numpy(slots[np.arange(n) // ps] * ps + np.arange(n) % ps).cuda().long()
+            pool = c.get_state(md.MD_STATE_POOL)
+            got = pool[:, :, :, 0].permute(0, 2, 1, 3, 4).reshape(L, Hkv, -1, 128)[:, :, at]
+            assert torch.equal(got, kd)
+            assert torch.equal(c.get_state(md.MD_STATE_REGION)[at].cpu(), torch.from_numpy(lab))
+            assert torch.equal(c.get_state(md.MD_STATE_T_INS)[at].cpu(), torch.from_numpy(step))
+        c.close()
+    for x, y in zip(*states):
+        assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("ps,aligned", [(16, 0), (32, 0), (16, 1), (32, 1)])
 @pytest.mark.parametrize("entry", ["device", "layers"])
 def test_append_inside_attention_writes_what_the_append_kernel_writes(ps, aligned, entry):
     """Decode steps whose attention launch appends the new tokens leave the
