@@ -1037,9 +1037,9 @@ MD_API md_status md_evict(md_ctx *c, int batch, const int32_t *budget, int32_t *
     if (budget[b] < 0) return fail(c, MD_ERR_INVALID_ARG, "negative budget");
   const int ps = cf.page_size;
 
-  /* stages 2-3 */
-  ScoreParams sp;
-  memset(&sp, 0, sizeof(sp));
+  ObserveParams op;
+  memset(&op, 0, sizeof(op));
+  ScoreParams &sp = op.s;
   sp.mass_acc = ptr<unsigned long long>(c, c->lay.mass_acc);
   sp.window = ptr<float>(c, c->lay.window);
   sp.a = ptr<float>(c, c->lay.a);
@@ -1075,55 +1075,70 @@ MD_API md_status md_evict(md_ctx *c, int batch, const int32_t *budget, int32_t *
   sp.keep_prio = 1;
   sp.reg = c->reg;
   sp.n_seqs = batch;
-  int tot = 0;
+  int tot = 0, most = 0;
   for (int b = 0; b < batch; ++b) {
     sp.n_tokens[b] = (int)c->n_tokens[b];
     sp.n_pages[b] = c->n_pages[b];
     sp.page_start[b] = tot;
     tot += c->n_pages[b];
+    most = std::max(most, c->n_pages[b]);
   }
   sp.page_start[batch] = tot;
   sp.total_pages = tot;
-  cudaEvent_t e0;
-  prof_begin(c, &e0);
-  cudaError_t e = launch_score(sp, c->stream);
-  prof_end(c, STAGE_SCORE, e0);
-  if (e != cudaSuccess) return cuda_fail(c, e, "score launch");
-
-  /* stage 4 */
-  SelectParams sel;
-  memset(&sel, 0, sizeof(sel));
-  sel.page_score = ptr<float>(c, c->lay.page_score);
-  sel.block_table = ptr<int32_t>(c, c->lay.block_table);
-  sel.free_stack = ptr<int32_t>(c, c->lay.free_stack);
-  sel.evict_list = ptr<int32_t>(c, c->lay.evict_list);
-  sel.user_evicted = evicted_ids_dev;
-  sel.page_fill = ptr<uint8_t>(c, c->lay.page_fill);
-  sel.seq_tokens = ptr<int32_t>(c, c->lay.seq_tokens);
-  sel.status = ptr<int>(c, c->lay.status);
-  sel.P_max = cf.max_pages_per_seq;
-  sel.n_seqs = batch;
-  sel.top = (int)c->m.free_top;
   bool warn = false;
   int any = 0, pushed = 0;
   std::vector<int> ev(batch);
   for (int b = 0; b < batch; ++b) {
-    const int P = c->n_pages[b];
-    const int want = std::max(0, P - budget[b]);
+    const int want = std::max(0, c->n_pages[b] - budget[b]);
     const int can = std::max(0, evictable_pages(c, b));
     ev[b] = std::min(want, can);
     if (ev[b] < want) warn = true;
-    sel.n_pages[b] = P;
-    sel.n_evict[b] = ev[b];
-    sel.push_off[b] = pushed;
+    op.n_evict[b] = ev[b];
+    op.push_off[b] = pushed;
     pushed += ev[b];
     any |= ev[b] > 0;
   }
-  if (any || evicted_ids_dev) {
+  const bool select = any || evicted_ids_dev;
+  cudaEvent_t e0;
+  cudaError_t e;
+  if (select && !sp.calib_on && most <= OBSERVE_PAGES && most * ps <= OBSERVE_SLOTS) {
+    op.block_table = ptr<int32_t>(c, c->lay.block_table);
+    op.free_stack = ptr<int32_t>(c, c->lay.free_stack);
+    op.user_evicted = evicted_ids_dev;
+    op.seq_tokens = ptr<int32_t>(c, c->lay.seq_tokens);
+    op.page_fill = ptr<uint8_t>(c, c->lay.page_fill);
+    op.status = ptr<int>(c, c->lay.status);
+    op.top = (int)c->m.free_top;
     prof_begin(c, &e0);
-    e = launch_select(sel, c->stream);
-    prof_end(c, STAGE_SELECT, e0);
-    if (e != cudaSuccess) return cuda_fail(c, e, "select launch");
+    e = launch_observe(op, c->stream);
+    prof_end(c, STAGE_SCORE, e0);
+    if (e != cudaSuccess) return cuda_fail(c, e, "observation launch");
+  } else {
+    prof_begin(c, &e0);
+    e = launch_score(sp, c->stream);
+    prof_end(c, STAGE_SCORE, e0);
+    if (e != cudaSuccess) return cuda_fail(c, e, "score launch");
+    if (select) {   /* stage 4 */
+      SelectParams sel;
+      sel.page_score = ptr<float>(c, c->lay.page_score);
+      sel.block_table = ptr<int32_t>(c, c->lay.block_table);
+      sel.free_stack = ptr<int32_t>(c, c->lay.free_stack);
+      sel.evict_list = ptr<int32_t>(c, c->lay.evict_list);
+      sel.user_evicted = evicted_ids_dev;
+      sel.page_fill = ptr<uint8_t>(c, c->lay.page_fill);
+      sel.seq_tokens = ptr<int32_t>(c, c->lay.seq_tokens);
+      sel.status = ptr<int>(c, c->lay.status);
+      sel.P_max = cf.max_pages_per_seq;
+      sel.n_seqs = batch;
+      sel.top = (int)c->m.free_top;
+      std::copy(op.n_evict, op.n_evict + batch, sel.n_evict);
+      std::copy(op.push_off, op.push_off + batch, sel.push_off);
+      std::copy(sp.n_pages, sp.n_pages + batch, sel.n_pages);
+      prof_begin(c, &e0);
+      e = launch_select(sel, c->stream);
+      prof_end(c, STAGE_SELECT, e0);
+      if (e != cudaSuccess) return cuda_fail(c, e, "select launch");
+    }
   }
   for (int b = 0; b < batch; ++b) {
     c->n_pages[b] -= ev[b];

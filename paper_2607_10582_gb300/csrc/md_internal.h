@@ -235,6 +235,22 @@ struct SelectParams {
 };
 cudaError_t launch_select(const SelectParams &p, cudaStream_t s);
 
+/* ----------------------------------------- observe (score and select) --- */
+/* Most pages and token slots of a sequence: a page's rank reads every key, and
+ * a block's 1,024 threads score 4,096 slots in four rounds (about 1 us each);
+ * beyond that the grid-wide score kernel is the faster one. */
+constexpr int OBSERVE_PAGES = 256, OBSERVE_SLOTS = 4096;
+struct ObserveParams {
+  ScoreParams s;                         // page_fill, seq_tokens: only with region-aligned pages
+  int32_t *block_table, *free_stack, *user_evicted, *seq_tokens;
+  uint8_t *page_fill;
+  int *status;
+  int top;
+  int n_evict[MD_MAX_BATCH];
+  int push_off[MD_MAX_BATCH];
+};
+cudaError_t launch_observe(const ObserveParams &p, cudaStream_t s);
+
 /* Launch of a kernel taking one parameter struct, with programmatic stream
  * serialization (the kernel calls pdl_wait() before touching global memory). */
 template <class P>

@@ -187,135 +187,140 @@ __device__ __forceinline__ float random_draw(unsigned long long seed, int t, siz
   return (float)(z >> 40) * 5.9604644775390625e-08f;
 }
 
-/* A tile is 32/PS consecutive pages, one lane per token slot, one warp per
- * tile; the loop count is uniform across the block so the segmented shuffle
- * reductions see every lane.  A token's step mass is one fixed-point
- * accumulator (the attention kernel adds every (layer, KV head) into it):
- * read and zeroed here, loaded together with the token's state.  The
- * launcher sizes the grid to one wave of resident blocks. */
+/* The calibration histogram of a block (Sec. IV-B, Eq. 6's input): observed
+ * mass in fixed point, so integer atomics keep the sums order-independent. */
+struct CalibSmem {
+  unsigned long long sum[8 * CALIB_BUCKETS];
+  unsigned int cnt[8 * CALIB_BUCKETS];
+};
+
+/* Stages 2-3 for one warp's tile of 32/PS consecutive pages, one lane per
+ * token slot: this lane's slot is `off` of page pg of sequence b (page_ok:
+ * there is such a page).  Returns the page's score, the same in all its lanes.
+ * A token's step mass is one fixed-point accumulator (the attention kernel
+ * adds every (layer, KV head) into it): read and zeroed here, loaded together
+ * with the token's state. */
+template <int PS>
+__device__ __forceinline__ float score_tile(const ScoreParams &p, int b, int pg, int off, bool page_ok, bool need_mass,
+                                            CalibSmem *calib) {
+  const float INF = INFINITY;
+  bool valid = false;
+  size_t slot = 0;
+  if (page_ok) {
+    valid = p.page_fill ? off < p.page_fill[(size_t)b * p.P_max + pg] : pg * PS + off < p.n_tokens[b];
+    slot = (size_t)p.block_table[(size_t)b * p.P_max + pg] * PS + off;
+  }
+  /* the token's state and its step mass, all loads independent */
+  int reg = 0, tr = 0, tins = 0, ntok = 1;
+  float a = 0.f, w = 0.f;
+  unsigned long long macc = 0ull;
+  if (valid) {
+    if (need_mass) macc = __ldcs(p.mass_acc + slot);
+    if (p.fold_only) {
+      w = p.window[slot];
+    } else {
+      reg = p.region[slot];
+      a = p.a[slot];
+      tr = p.t_ref[slot];
+      if (p.observe) w = p.window[slot];
+      if (p.observe || p.score_mode == 2) ntok = p.seq_tokens ? p.seq_tokens[b] : p.n_tokens[b];
+      if (calib || p.score_mode == 3) tins = p.t_ins[slot];
+    }
+  }
+  /* the sum over layers and query heads, rounded once to fp32 */
+  const float msum = __ull2float_rn(macc) * MASS_UNIT;
+  if (valid && need_mass) p.mass_acc[slot] = 0ull;
+  float s = 0.f;
+  int pinned = 0;
+  if (valid) {
+    if (p.fold_only) {
+      p.window[slot] = w + msum;
+    } else {
+      if (p.observe) {
+        if (p.mass_pending) w += msum;
+        const float abar = __fdiv_rn(w, p.norm);                    // Sec. III-C
+        a = p.rho * a + p.gamma * abar;                             // Eq. 2
+        const float tau = __fdiv_rn(p.tau_scale, (float)ntok);
+        if (abar >= tau) tr = p.t;                                  // Eq. 3
+        p.window[slot] = 0.f;
+        p.ahat[slot] = abar;
+        p.a[slot] = a;
+        p.t_ref[slot] = tr;
+        if (calib) {
+          const int age = p.t - tins;
+          const int bkt = age >= 0 ? age / CALIB_WIDTH : -1;
+          if (bkt >= 0 && bkt < CALIB_BUCKETS) {
+            atomicAdd(&calib->sum[reg * CALIB_BUCKETS + bkt], __float2ull_rn(abar * 4294967296.0f));
+            atomicAdd(&calib->cnt[reg * CALIB_BUCKETS + bkt], 1u);
+          }
+        }
+      }
+      const float x = __fdiv_rn((float)(p.t - tr), p.reg.half_life[reg]);
+      const float d = exp2f(-x);                                    // Eqs. 4, 7
+      switch (p.score_mode) {
+        case 0: s = p.reg.base[reg] * d + p.alpha * a; break;       // Eq. 4
+        case 1: s = (p.reg.base[reg] + p.alpha * a) * d; break;
+        case 2: s = p.reg.base[reg] * d + p.alpha * a * (float)ntok; break;
+        case 3: s = (float)tins; break;                             // recency
+        default: s = random_draw(p.random_seed, p.t, slot); break;   // random
+      }
+      pinned = p.reg.pinned[reg];
+      if (pinned) s = INF;
+      if (p.keep_prio) p.prio[slot] = s;
+    }
+  }
+  if (p.fold_only) return 0.f;
+  float sum = (valid && !pinned) ? s : 0.f;
+  float mx = (valid && !pinned) ? s : -INF;
+  int anyp = (valid && pinned) ? 1 : 0;
+  int cnt = valid ? 1 : 0;
+#pragma unroll
+  for (int o = PS / 2; o > 0; o >>= 1) {
+    sum += __shfl_xor_sync(0xffffffffu, sum, o, PS);
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o, PS));
+    anyp |= __shfl_xor_sync(0xffffffffu, anyp, o, PS);
+    cnt += __shfl_xor_sync(0xffffffffu, cnt, o, PS);
+  }
+  float S = INF;                                                   // pinning, tail
+  if (page_ok && !anyp && pg != p.n_pages[b] - 1)
+    S = (p.page_reduce == 0) ? __fdiv_rn(sum, (float)cnt) : mx;   // Eq. 5
+  if (page_ok && off == 0) p.page_score[(size_t)b * p.P_max + pg] = S;
+  return S;
+}
+
+/* One warp per tile; the loop count is uniform across a warp, so the segmented
+ * shuffle reductions see every lane.  The launcher sizes the grid to one wave
+ * of resident blocks. */
 template <int PS>
 __global__ void __launch_bounds__(256, 6) score_kernel(const __grid_constant__ ScoreParams p) {
   pdl_wait();
   pdl_trigger();
   constexpr int PPW = 32 / PS;
-  /* calibration histogram of this block (Sec. IV-B, Eq. 6's input): observed
-   * mass in fixed point, so integer atomics keep the sums order-independent */
-  __shared__ unsigned long long h_sum[8 * CALIB_BUCKETS];
-  __shared__ unsigned int h_cnt[8 * CALIB_BUCKETS];
+  __shared__ CalibSmem hist;
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   const int tiles = (p.total_pages + PPW - 1) / PPW;
   const bool need_mass = p.fold_only || (p.observe && p.mass_pending);
-  const float INF = INFINITY;
   const bool calib = p.calib_on && p.observe && !p.fold_only;
   if (calib) {
     for (int k = threadIdx.x; k < 8 * CALIB_BUCKETS; k += blockDim.x) {
-      h_sum[k] = 0ull;
-      h_cnt[k] = 0u;
+      hist.sum[k] = 0ull;
+      hist.cnt[k] = 0u;
     }
     __syncthreads();
   }
   for (int t0 = blockIdx.x * 8; t0 < tiles; t0 += gridDim.x * 8) {
-    const int base = (t0 + wib) * PPW;
-    const int gp = base + lane / PS;
-    const int off = lane % PS;
+    const int gp = (t0 + wib) * PPW + lane / PS;
     const bool page_ok = gp < p.total_pages;
-    int b = 0, pg = 0, P = 0;
-    bool valid = false;
-    size_t slot = 0;
-    if (page_ok) {
-      b = find_seq(p.page_start, p.n_seqs, gp);
-      pg = gp - p.page_start[b];
-      P = p.n_pages[b];
-      valid = p.page_fill ? off < p.page_fill[(size_t)b * p.P_max + pg]
-                          : pg * PS + off < p.n_tokens[b];
-      slot = (size_t)p.block_table[(size_t)b * p.P_max + pg] * PS + off;
-    }
-    /* the token's state and its step mass, all loads independent */
-    int reg = 0, tr = 0, tins = 0, ntok = 1;
-    float a = 0.f, w = 0.f;
-    unsigned long long macc = 0ull;
-    if (valid) {
-      if (need_mass) macc = __ldcs(p.mass_acc + slot);
-      if (p.fold_only) {
-        w = p.window[slot];
-      } else {
-        reg = p.region[slot];
-        a = p.a[slot];
-        tr = p.t_ref[slot];
-        if (p.observe) w = p.window[slot];
-        if (p.observe || p.score_mode == 2) ntok = p.seq_tokens ? p.seq_tokens[b] : p.n_tokens[b];
-        if (calib || p.score_mode == 3) tins = p.t_ins[slot];
-      }
-    }
-    /* the sum over layers and query heads, rounded once to fp32 */
-    const float msum = __ull2float_rn(macc) * MASS_UNIT;
-    if (valid && need_mass) p.mass_acc[slot] = 0ull;
-    float s = 0.f;
-    int pinned = 0;
-    if (valid) {
-      if (p.fold_only) {
-        p.window[slot] = w + msum;
-      } else {
-        if (p.observe) {
-          if (p.mass_pending) w += msum;
-          const float abar = __fdiv_rn(w, p.norm);                    // Sec. III-C
-          a = p.rho * a + p.gamma * abar;                             // Eq. 2
-          const float tau = __fdiv_rn(p.tau_scale, (float)ntok);
-          if (abar >= tau) tr = p.t;                                  // Eq. 3
-          p.window[slot] = 0.f;
-          p.ahat[slot] = abar;
-          p.a[slot] = a;
-          p.t_ref[slot] = tr;
-          if (calib) {
-            const int age = p.t - tins;
-            const int bkt = age >= 0 ? age / CALIB_WIDTH : -1;
-            if (bkt >= 0 && bkt < CALIB_BUCKETS) {
-              atomicAdd(&h_sum[reg * CALIB_BUCKETS + bkt], __float2ull_rn(abar * 4294967296.0f));
-              atomicAdd(&h_cnt[reg * CALIB_BUCKETS + bkt], 1u);
-            }
-          }
-        }
-        const float x = __fdiv_rn((float)(p.t - tr), p.reg.half_life[reg]);
-        const float d = exp2f(-x);                                    // Eqs. 4, 7
-        switch (p.score_mode) {
-          case 0: s = p.reg.base[reg] * d + p.alpha * a; break;       // Eq. 4
-          case 1: s = (p.reg.base[reg] + p.alpha * a) * d; break;
-          case 2: s = p.reg.base[reg] * d + p.alpha * a * (float)ntok; break;
-          case 3: s = (float)tins; break;                             // recency
-          default: s = random_draw(p.random_seed, p.t, slot); break;   // random
-        }
-        pinned = p.reg.pinned[reg];
-        if (pinned) s = INF;
-        if (p.keep_prio) p.prio[slot] = s;
-      }
-    }
-    if (!p.fold_only) {
-      float sum = (valid && !pinned) ? s : 0.f;
-      float mx = (valid && !pinned) ? s : -INF;
-      int anyp = (valid && pinned) ? 1 : 0;
-      int cnt = valid ? 1 : 0;
-#pragma unroll
-      for (int o = PS / 2; o > 0; o >>= 1) {
-        sum += __shfl_xor_sync(0xffffffffu, sum, o, PS);
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o, PS));
-        anyp |= __shfl_xor_sync(0xffffffffu, anyp, o, PS);
-        cnt += __shfl_xor_sync(0xffffffffu, cnt, o, PS);
-      }
-      if (page_ok && off == 0) {
-        float S;
-        if (anyp || pg == P - 1) S = INF;                            // pinning, tail
-        else S = (p.page_reduce == 0) ? __fdiv_rn(sum, (float)cnt) : mx;   // Eq. 5
-        p.page_score[(size_t)b * p.P_max + pg] = S;
-      }
-    }
+    const int b = page_ok ? find_seq(p.page_start, p.n_seqs, gp) : 0;
+    score_tile<PS>(p, b, page_ok ? gp - p.page_start[b] : 0, lane % PS, page_ok, need_mass, calib ? &hist : nullptr);
   }
   if (calib) {
     __syncthreads();
     for (int k = threadIdx.x; k < 8 * CALIB_BUCKETS; k += blockDim.x)
-      if (h_cnt[k]) {
-        atomicAdd(&p.calib_sum[k], h_sum[k]);
-        atomicAdd(&p.calib_cnt[k], h_cnt[k]);
+      if (hist.cnt[k]) {
+        atomicAdd(&p.calib_sum[k], hist.sum[k]);
+        atomicAdd(&p.calib_cnt[k], hist.cnt[k]);
       }
   }
 }
@@ -526,6 +531,95 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const __grid_consta
   }
   if (uout)
     for (int i = e + threadIdx.x; i < p.P_max; i += blockDim.x) uout[i] = -1;
+}
+
+/* Stages 2-4 in one launch for short sequences (at most OBSERVE_PAGES pages):
+ * one block scores its sequence's pages and then selects among them in shared
+ * memory.  What bounds a short observation is the chain of dependent launches
+ * and round trips, not the bytes: a decode step of 32 sequences of 430 tokens
+ * and its observation took 102.3 us with the two kernels and their hand-over
+ * through the page-score array, 97.9 with this one.  With so few keys a page's rank is counted directly (one thread per
+ * page reads every key, a broadcast), instead of up to four radix passes of
+ * three barriers each; ties go to the lower logical index as there. */
+template <int PS>
+__global__ void __launch_bounds__(1024) observe_kernel(const __grid_constant__ ObserveParams p) {
+  __shared__ __align__(16) uint32_t keys[OBSERVE_PAGES];
+  __shared__ int warp_ev[OBSERVE_PAGES / 32];
+  __shared__ int s_gone;
+  pdl_wait();
+  pdl_trigger();
+  constexpr int PPW = 32 / PS;
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int P = p.s.n_pages[b], e = p.n_evict[b];
+  int32_t *row = p.block_table + (size_t)b * p.s.P_max;
+  uint8_t *frow = p.page_fill + (size_t)b * p.s.P_max;
+  int32_t *uout = p.user_evicted ? p.user_evicted + (size_t)b * p.s.P_max : nullptr;
+  /* thread i < P: page i's id and fill, before anything is compacted */
+  const int id = tid < P ? row[tid] : 0, fill = tid < P ? frow[tid] : 0;
+  if (tid == 0) s_gone = 0;
+  if (tid < OBSERVE_PAGES && tid >= P) keys[tid] = KEY_PINNED;
+  for (int pg0 = warp * PPW; pg0 < P; pg0 += (int)(blockDim.x >> 5) * PPW) {
+    const int pg = pg0 + lane / PS;
+    const float S = score_tile<PS>(p.s, b, pg < P ? pg : 0, lane % PS, pg < P, p.s.observe && p.s.mass_pending, nullptr);
+    if (pg < P && lane % PS == 0) keys[pg] = S == INFINITY ? KEY_PINNED : order_key(S);
+  }
+  __syncthreads();
+  if (e > 0) {
+    /* page tid's rank among the evictable pages: keys below its own, and
+     * equal ones at lower indices */
+    const int P4 = (P + 3) / 4;
+    int ev = 0;
+    if (tid < P) {
+      const uint32_t k = keys[tid];
+      int rank = 0;
+      for (int j = 0; j < P4; ++j) {
+        const uint4 q = ((const uint4 *)keys)[j];
+        const int i = 4 * j;
+        rank += (q.x < k || (q.x == k && i < tid)) + (q.y < k || (q.y == k && i + 1 < tid)) +
+                (q.z < k || (q.z == k && i + 2 < tid)) + (q.w < k || (q.w == k && i + 3 < tid));
+      }
+      ev = k != KEY_PINNED && rank < e;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, ev);
+    if (lane == 0 && warp < OBSERVE_PAGES / 32) warp_ev[warp] = __popc(m);
+    __syncthreads();
+    int idx = __popc(m & ((1u << lane) - 1)), total = 0;
+    for (int w = 0; w < (P + 31) / 32; ++w) {
+      idx += w < warp ? warp_ev[w] : 0;
+      total += warp_ev[w];
+    }
+    if (total != e) {   // fewer evictable pages than e: nothing is changed
+      if (tid == 0) atomicCAS(&p.status[ST_CODE], 0, (int)MD_ERR_STATE);
+      return;
+    }
+    if (tid < P) {
+      if (ev) {
+        p.free_stack[p.top + p.push_off[b] + idx] = id;
+        if (uout) uout[idx] = id;
+        atomicAdd(&s_gone, fill);
+      } else {
+        row[tid - idx] = id;
+        frow[tid - idx] = (uint8_t)fill;
+      }
+    }
+    __syncthreads();
+    if (tid == 0) p.seq_tokens[b] -= s_gone;
+    if (tid < P && tid >= P - e) {
+      row[tid] = -1;
+      frow[tid] = 0;
+    }
+  }
+  if (uout)
+    for (int i = e + tid; i < p.s.P_max; i += blockDim.x) uout[i] = -1;
+}
+
+cudaError_t launch_observe(const ObserveParams &p, cudaStream_t s) {
+  int pmax = 1;
+  for (int b = 0; b < p.s.n_seqs; ++b) pmax = p.s.n_pages[b] > pmax ? p.s.n_pages[b] : pmax;
+  int threads = (pmax * p.s.ps + 31) / 32 * 32;   // one token slot per thread, up to a full block
+  threads = threads > 1024 ? 1024 : threads;
+  return p.s.ps == 16 ? launch_pdl(observe_kernel<16>, p.s.n_seqs, threads, 0, s, p)
+                      : launch_pdl(observe_kernel<32>, p.s.n_seqs, threads, 0, s, p);
 }
 
 cudaError_t launch_select(const SelectParams &p, cudaStream_t s) {

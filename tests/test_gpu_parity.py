@@ -447,6 +447,50 @@ def test_output_at_any_address(n):
     assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
 
 
+@pytest.mark.parametrize("ps,aligned,reduce", [(16, 0, 0), (32, 0, 1), (16, 1, 1), (32, 1, 0)])
+def test_one_launch_observation_selects_what_the_two_kernels_select(ps, aligned, reduce):
+    """A batch of short sequences, scored and selected in one launch, against
+    the same batch with the calibration histogram on, which takes the two
+    kernels: token state, page scores, tables, fills, counts and evicted pages
+    bit for bit.  Pages at the ends of warps and of the kernel's range, none,
+    one, several and all evictable pages evicted, equal scores (b = 0 and no
+    attention weight)."""
+    sizes = [1, ps, 31 * ps, 32 * ps, 33 * ps - 1, 4096 // ps * ps - 2, 70 * ps + 5, 5 * ps]
+    cut = [0, 1, 1, 31, 17, 90, 200, 99]
+    B = len(sizes)
+    for weight in (1.0, 0.0):
+        got = []
+        for two_kernels in (False, True):
+            c = md.Cache(1, 4, 1, ps, B, 700, 700 * B, page_reduce=reduce, attn_weight=weight,
+                         region_aligned_pages=aligned)
+            for r in range(7):
+                c.set_region_params(r, 0.0 if weight == 0.0 else 0.3 + 0.1 * r, 20.0, r == 0)
+            for b, m in enumerate(sizes):
+                lab = (np.arange(m) // 23 % 7).astype(np.uint8)
+                k, v = synth.kv_host(19, b, 1, 1, 0, m, lab)
+                c.append_tokens(b, lab, to_dev(k), to_dev(v), -(np.arange(m, dtype=np.int32)[::-1] // 40))
+            c.calib_enable(two_kernels)
+            q = synth.q_host(19, B, 1, 4, 1, 1)
+            kn, vn = synth.step_kv_host(19, sizes, [6] * B, 1, 1)
+            out = torch.empty((B, 1, 4, 128), dtype=torch.int16, device="cuda")
+            c.decode_step(B, to_dev(q), to_dev(kn), to_dev(vn), [6] * B, out)
+            pages = [c.query(md.MD_QUERY_PAGES, b) for b in range(B)]
+            ids = torch.full((B, 700), -7, dtype=torch.int32, device="cuda")
+            before = c.get_state(md.MD_STATE_BLOCK_TABLE)
+            st, n_ev = c.evict([max(0, p - e) for p, e in zip(pages, cut)], ids)
+            assert c.sync() == md.MD_OK
+            got.append([before, torch.from_numpy(n_ev), ids] + [c.get_state(w) for w in (
+                md.MD_STATE_PAGE_SCORE, md.MD_STATE_BLOCK_TABLE, md.MD_STATE_PAGE_FILL, md.MD_STATE_SEQ_TOKENS)])
+            slot = before.cpu().numpy()
+            slot = torch.from_numpy(np.concatenate([slot[b, :pages[b]] for b in range(B)]).astype(np.int64)).cuda()
+            got[-1] += [c.get_state(w).view(-1, ps)[slot] for w in (
+                md.MD_STATE_A, md.MD_STATE_T_REF, md.MD_STATE_AHAT, md.MD_STATE_TOKEN_PRIO, md.MD_STATE_WINDOW)]
+            c.close()
+        assert int(got[0][1].sum()) > 100
+        for x, y in zip(*got):
+            assert torch.equal(x, y)
+
+
 @pytest.mark.parametrize("ps,aligned", [(16, 0), (32, 0), (16, 1), (32, 1)])
 @pytest.mark.parametrize("runs", ["spans", "single tokens"])
 def test_append_in_one_call_and_in_pieces(ps, aligned, runs):
