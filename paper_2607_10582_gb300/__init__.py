@@ -4,7 +4,9 @@ Python binding of ``include/memdecay.h``: the same calls, argument
 marshalling only.  Every step of the path runs in the CUDA kernels of
 ``libmemdecay.so``; there is no CPU or PyTorch fallback, and importing the
 binding fails loudly when the library has not been built.  PyTorch provides
-device memory (the workspace, input and output tensors) and streams.
+device memory (the workspace, input and output tensors) and streams.  The
+calls of a decode loop go through a small C module (csrc/md_binding.c); the
+others, and arguments it does not take in place, through ctypes.
 """
 from __future__ import annotations
 
@@ -116,6 +118,24 @@ def lib():
     return _lib
 
 
+_fast = None
+
+
+def _binding():
+    """The C module of the per-step calls, bound to the library.  Raises if it
+    has not been built."""
+    global _fast
+    if _fast is None:
+        lib()
+        try:
+            from . import _calls as m
+        except ImportError as e:
+            raise RuntimeError("_calls.so is missing: build it with `python -m paper_2607_10582_gb300.build`") from e
+        m.load(LIB_PATH)
+        _fast = m
+    return _fast
+
+
 class MemDecayError(RuntimeError):
     def __init__(self, status: int, msg: str):
         super().__init__(f"{STATUS_NAMES.get(status, status)}: {msg}")
@@ -199,10 +219,11 @@ class Cache:
         h = ctypes.c_void_p()
         self._check(lib().md_create(ctypes.byref(c), ctypes.byref(h)), None)
         self.h = h
+        self._b, self._hv, self._specs = _binding(), h.value, self._state_specs()
 
     # -- plumbing --
     def _check(self, st: int, h=0, ok=(MD_OK,)):
-        if st in ok:
+        if st == MD_OK or st in ok:
             return st
         msg = ""
         if h is not None:
@@ -214,6 +235,7 @@ class Cache:
         if getattr(self, "h", None):
             lib().md_destroy(self.h)
             self.h = None
+            self._hv = None
 
     def __del__(self):
         try:
@@ -233,6 +255,9 @@ class Cache:
         return self._check(lib().md_append_tokens(self.h, seq, len(regs), rp, sp, _ptr(k), _ptr(v)))
 
     def decode_step(self, batch: int, q, k_new, v_new, new_regions, out):
+        st = self._b.decode_step(self._hv, batch, q, k_new, v_new, new_regions, out)
+        if st is not None:
+            return self._check(st)
         regs, rp = _host(new_regions, np.uint8)
         return self._check(lib().md_decode_step(self.h, batch, _ptr(q), _ptr(k_new), _ptr(v_new), rp, _ptr(out)))
 
@@ -240,19 +265,30 @@ class Cache:
         """md_decode_step_host: q, k_new, v_new and out are host buffers (CPU
         tensors or numpy arrays, bf16 bits); out is written once the stream
         gets there (sync() or a stream synchronisation)."""
+        st = self._b.decode_step_host(self._hv, batch, q, k_new, v_new, new_regions, out)
+        if st is not None:
+            return self._check(st)
         regs, rp = _host(new_regions, np.uint8)
         return self._check(lib().md_decode_step_host(self.h, batch, _hptr(q), _hptr(k_new), _hptr(v_new), rp,
                                                      _hptr(out)))
 
     def decode_layer(self, layer: int, batch: int, q, k_new, v_new, new_regions, out):
+        st = self._b.decode_layer(self._hv, layer, batch, q, k_new, v_new, new_regions, out)
+        if st is not None:
+            return self._check(st)
         regs, rp = _host(new_regions, np.uint8)
         return self._check(lib().md_decode_layer(self.h, layer, batch, _ptr(q), _ptr(k_new), _ptr(v_new), rp,
                                                  _ptr(out)))
 
     def evict(self, budgets: Sequence[int], evicted_ids=None):
-        bud, bp = _host(budgets, np.int32)
-        n_ev = np.zeros(len(bud), np.int32)
-        st = lib().md_evict(self.h, len(bud), bp, n_ev.ctypes.data, _ptr(evicted_ids))
+        st = None
+        if type(budgets) is np.ndarray and budgets.ndim == 1:
+            n_ev = np.zeros(len(budgets), np.int32)
+            st = self._b.evict(self._hv, budgets, n_ev, evicted_ids)
+        if st is None:
+            bud, bp = _host(budgets, np.int32)
+            n_ev = np.zeros(len(bud), np.int32)
+            st = lib().md_evict(self.h, len(bud), bp, n_ev.ctypes.data, _ptr(evicted_ids))
         self._check(st, 0, ok=(MD_OK, MD_WARN_OVER_BUDGET))
         return st, n_ev
 
@@ -264,7 +300,7 @@ class Cache:
         self._check(lib().md_query(self.h, what, seq, ctypes.byref(v)))
         return int(v.value)
 
-    def state_spec(self, what: int):
+    def _state_specs(self):
         slots = self.P_phys * self.ps
         t = self.torch
         return {
@@ -283,12 +319,16 @@ class Cache:
             MD_STATE_PAGE_FILL: ((self.max_batch, self.P_max), t.uint8),
             MD_STATE_SEQ_TOKENS: ((self.max_batch,), t.int32),
             MD_STATE_CALIB: ((8 * MD_CALIB_BUCKETS * 12,), t.uint8),
-        }[what]
+        }
+
+    def state_spec(self, what: int):
+        """(shape, dtype) of a state array."""
+        return self._specs[what]
 
     def get_state(self, what: int):
-        shape, dt = self.state_spec(what)
+        shape, dt = self._specs[what]
         out = self.torch.empty(shape, dtype=dt, device=self.device)
-        self._check(lib().md_get_state(self.h, what, out.data_ptr(), out.numel() * out.element_size()))
+        self._check(self._b.get_state(self._hv, what, out, out.nbytes))
         return out
 
     def set_state(self, what: int, src):

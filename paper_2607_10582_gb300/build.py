@@ -1,18 +1,21 @@
 """In-tree build of libmemdecay.so for sm_103a (nvcc; no cmake).
 
 The translation units compile in parallel, then link into one shared library
-next to this file.  Run as a module or call build()."""
+next to this file; the Python module of the per-step calls (_calls.so, plain
+C) lands beside it.  Run as a module or call build()."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB_PATH = os.path.join(HERE, "libmemdecay.so")
+BINDING_PATH = os.path.join(HERE, "_calls.so")
 OBJ_DIR = os.path.join(HERE, "_build")
 SOURCES = ["md_host.cpp", "md_attn.cu", "md_attn_cluster.cu", "md_state.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -29,7 +32,7 @@ def _deps():
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) -> str:
     newest = max(os.path.getmtime(p) for p in _deps())
-    if not force and os.path.exists(LIB_PATH) and os.path.getmtime(LIB_PATH) >= newest:
+    if not force and all(os.path.exists(p) and os.path.getmtime(p) >= newest for p in (LIB_PATH, BINDING_PATH)):
         return LIB_PATH
     os.makedirs(OBJ_DIR, exist_ok=True)
 
@@ -47,8 +50,18 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
             raise RuntimeError(f"nvcc failed on {src}")
         return obj
 
-    with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    def compile_binding():
+        cmd = ["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", INCLUDE,
+               os.path.join(CSRC, "md_binding.c"), "-o", BINDING_PATH + ".tmp", "-ldl"]
+        if verbose:
+            print(" ".join(cmd), flush=True)
+        subprocess.run(cmd, check=True)
+        os.replace(BINDING_PATH + ".tmp", BINDING_PATH)
+
+    with ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
+        binding = ex.submit(compile_binding)
         objs = list(ex.map(compile_one, SOURCES))
+        binding.result()
     tmp = LIB_PATH + ".tmp"
     cmd = ["nvcc", *ARCH, "-shared", "-o", tmp, *objs, "-cudart", "static"]
     if verbose:

@@ -581,6 +581,52 @@ def test_append_inside_attention_writes_what_the_append_kernel_writes(ps, aligne
         c.close()
 
 
+def test_argument_forms_give_the_same_step():
+    """Labels and budgets as exact arrays (taken in place), lists, other
+    integer types and strided arrays; host buffers as tensors and as numpy
+    arrays: the same outputs and counts."""
+    L, Hq, Hkv, ps, n = 2, 8, 2, 16, [100, 333]
+    q = synth.q_host(23, 2, L, Hq, Hkv, 1)
+    kn, vn = synth.step_kv_host(23, n, [5, 6], L, Hkv)
+    forms = [np.array([5, 6], np.uint8), [5, 6], np.array([5, 6], np.int64), np.array([5, 9, 6, 9], np.uint8)[::2]]
+    cuts = [np.array([4, 9], np.int32), [4, 9], np.array([4, 9], np.int64), np.array([4, 0, 9, 0], np.int32)[::2]]
+    seen = []
+    for entry in ("device", "layers", "host tensors", "host arrays"):
+        for regs, cut in zip(forms, cuts):
+            c = md.Cache(L, Hq, Hkv, ps, 2, 30, 60)
+            for b, m in enumerate(n):
+                k, v = synth.kv_host(23, b, L, Hkv, 0, m)
+                c.append_tokens(b, np.full(m, 4, np.uint8), to_dev(k), to_dev(v))
+            out = torch.empty((2, L, Hq, 128), dtype=torch.int16, device="cuda")
+            if entry == "device":
+                c.decode_step(2, to_dev(q), to_dev(kn), to_dev(vn), regs, out)
+            elif entry == "layers":
+                for l in range(L):
+                    o = torch.empty((2, Hq, 128), dtype=torch.int16, device="cuda")
+                    c.decode_layer(l, 2, to_dev(q[:, l]), to_dev(kn[:, l]), to_dev(vn[:, l]), regs, o)
+                    out[:, l] = o
+            else:
+                host = [np.ascontiguousarray(a).view(np.int16) for a in (q, kn, vn)]
+                res = np.zeros((2, L, Hq, 128), np.int16)
+                if entry == "host tensors":
+                    c.decode_step_host(2, *[torch.from_numpy(a) for a in host], regs, torch.from_numpy(res))
+                else:
+                    c.decode_step_host(2, *host, regs, res)
+                assert c.sync() == md.MD_OK
+                out = torch.from_numpy(res).cuda()
+            st, n_ev = c.evict(cut)
+            assert st == md.MD_OK and n_ev.dtype == np.int32 and list(n_ev) == [3, 12]
+            seen.append((out.clone(), c.get_state(md.MD_STATE_REGION), c.get_state(md.MD_STATE_BLOCK_TABLE)))
+            with pytest.raises(md.MemDecayError):
+                c.decode_step(3, 1, 1, 1, regs, 1)
+            c.close()
+    x = synth.bf16_to_f64(seen[0][0].cpu().numpy().view(np.uint16))
+    for o, reg, tab in seen[1:]:
+        y = synth.bf16_to_f64(o.cpu().numpy().view(np.uint16))
+        assert np.max(np.abs(x - y)) <= TOL_O_ABS
+        assert torch.equal(reg, seen[0][1]) and torch.equal(tab, seen[0][2])
+
+
 def test_checkpoint_restore_replays_step():
     w = synth.custom_workload("ckpt", L=2, Hq=8, Hkv=2, page_size=16, lengths=[900],
                               budget_frac=0.3, steps=2, seed=9)
