@@ -1216,10 +1216,10 @@ extern "C" __attribute__((visibility("default"))) md_status md_attend_mass_noall
   CUtensorMap tmap;
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e;
-  const ClusterPlan plan = cluster_plan(ap);
+  const ClusterPlan plan = cluster_plan(ap, 0);
   if (plan.C > 0) {   // needs no scratch: nothing of the array is touched
     if (!encode_tile_map(encode, &tmap, (void *)kv_pool_dev, rows, ps)) return MD_ERR_INVALID_ARG;
-    e = launch_cluster(ap, plan, false, tmap, st);
+    e = launch_cluster(ap, plan, false, nullptr, tmap, st);
     return e == cudaSuccess ? MD_OK : MD_ERR_CUDA;
   }
   if (!encode_page_map(encode, &tmap, (void *)kv_pool_dev, rows, ps)) return MD_ERR_INVALID_ARG;

@@ -13,6 +13,8 @@
  *   - every chunk pushes its (m, Z) and the slices of its O into the shared
  *     memory of the item's other CTAs; after one cluster barrier each CTA has
  *     everything for its slice of the output and its own tokens' masses.
+ * LONG: chunks whose scores do not fit shared memory keep them in the
+ * workspace's scratch (L2), and a lane's page ids are loaded 32 tiles at a time.
  * A cluster's CTAs are co-scheduled by the hardware, so nothing polls; the
  * only software waits are the bounded ones on the CTA's own copies. */
 #include <cuda_bf16.h>
@@ -35,23 +37,25 @@ constexpr int misc_bytes(int warps) { return warps * STAGES * 8 + (2 * warps * G
 /* from every CTA of the cluster: (m, Z) per head, its O over this CTA's slice */
 constexpr int XCH_BYTES = (MAX_CLUSTER * GP * 2 + GP * D) * 4;
 constexpr int CLUSTER_SMEM = 227 * 1024, SM_SMEM = 228 * 1024;   // most a block may have, an SM has
+constexpr double LONG_SCORES = 48e6;              // most bytes of spilled scores (L2 is 129 MB, K/V stream through it)
 static_assert(GP * OS * 4 <= TILE_BYTES, "a warp's O^T fits one of its stages");
 static_assert(D % (8 * MAX_CLUSTER) == 0, "8 consecutive elements of O lie in one slice");
 
 }  // namespace
 
+/* warp_tiles: tiles per warp whose scores are kept here (LONG: 0) */
 static size_t cluster_smem(int warps, int C, int warp_tiles) {
   return 1024 + (size_t)warps * (STAGES * TILE_BYTES + warp_tiles * SCORE_BYTES) + misc_bytes(warps) +
          (C > 1 ? XCH_BYTES : 0);
 }
 
-template <bool ALIGNED, bool ROWS, int NW>
+template <bool ALIGNED, bool ROWS, int NW, bool LONG>
 __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
     attn_cluster_kernel(const __grid_constant__ ClusterParams p, const __grid_constant__ CUtensorMap tmap) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *ring = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   float *scores = (float *)(ring + NW * STAGES * TILE_BYTES);
-  float *wm = scores + (size_t)NW * p.warp_tiles * TILE * GP;
+  float *wm = scores + (LONG ? 0 : (size_t)NW * p.warp_tiles * TILE * GP);
   float *wl = wm + NW * GP;
   float *fin = wl + NW * GP;      // [16] the item's per-head max, then 1/Z (one chunk per item)
   uint64_t *full = (uint64_t *)(fin + 2 * GP);
@@ -90,24 +94,30 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
    * tiles of all pages, each masked by its page's fill */
   const int tiles = ALIGNED ? (last + 1) * tpp : (n_tok + TILE - 1) / TILE;
   const int t0 = (int)((long long)rank * tiles / C), t1 = (int)((long long)(rank + 1) * tiles / C);
-  const int nt = t1 - t0 > warp ? (t1 - t0 - warp + NW - 1) / NW : 0;   // this warp's tiles, at most 32
+  const int nt = t1 - t0 > warp ? (t1 - t0 - warp + NW - 1) / NW : 0;   // this warp's tiles (not LONG: at most 32)
 
-  /* Lane n keeps the page id and the token count of the warp's n-th tile.
+  /* Lane i keeps the page id and the token count of the warp's tile i (LONG:
+   * 32 k + i, and id2, fill2 those of the next 32).
    * Layers after a step's first one only read pages and table entries that
    * were complete before that first layer's launch (the new token's own rows
    * and table entry come from the launch parameters), so their K/V copies
    * start before the kernel ahead has finished. */
   if (!p.early) pdl_wait();
-  int id = 0, fill = 0;
-  const int my_tile = t0 + warp + NW * lane;
-  if (lane < nt) {
-    const int pg = my_tile >> shift;
-    id = *(pop >= 0 && pg == last ? p.nt.free_stack + pop : p.block_table + (size_t)b * p.P_max + pg);
-    if (ALIGNED)
-      fill = (add && pg == last ? tail_fill : p.page_fill[(size_t)b * p.P_max + pg]) - (my_tile & (tpp - 1)) * TILE;
-    else
-      fill = n_tok - my_tile * TILE;
-  }
+  auto load_ids = [&](int n0, int &page, int &valid) {   // of tiles n0 .. n0 + 31
+    page = valid = 0;
+    const int tile = t0 + warp + NW * (n0 + lane);
+    if (n0 + lane < nt) {
+      const int pg = tile >> shift;
+      page = *(pop >= 0 && pg == last ? p.nt.free_stack + pop : p.block_table + (size_t)b * p.P_max + pg);
+      if (ALIGNED)
+        valid = (add && pg == last ? tail_fill : p.page_fill[(size_t)b * p.P_max + pg]) - (tile & (tpp - 1)) * TILE;
+      else
+        valid = n_tok - tile * TILE;
+    }
+  };
+  int id, fill, id2 = 0, fill2 = 0;
+  load_ids(0, id, fill);
+  if (LONG) load_ids(32, id2, fill2);
   const uint64_t pol = policy_evict_first();
   auto copy_tile = [&](int n, int tile, int page) {
     const uint32_t st = ring_u32 + (n % STAGES) * TILE_BYTES, bar = bar_u32 + (n % STAGES) * 8;
@@ -117,7 +127,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
     tma_load_4d(st + HALF_BYTES, &tmap, 64, y, 0, row, bar, pol);
   };
   if (p.early) {
-    if (lane < STAGES && lane < nt) copy_tile(lane, my_tile, id);
+    if (lane < STAGES && lane < nt) copy_tile(lane, t0 + warp + NW * lane, id);
     pdl_wait();
   }
   pdl_trigger();
@@ -133,7 +143,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
       qf[kk][1] = g < G ? *(const uint32_t *)(qrow + 16 * kk + 8) : 0u;
     }
   }
-  if (!p.early && lane < STAGES && lane < nt) copy_tile(lane, my_tile, id);
+  if (!p.early && lane < STAGES && lane < nt) copy_tile(lane, t0 + warp + NW * lane, id);
   /* the new token's rows (16 bytes per lane: K, then V), if this warp has its tile */
   int n_tail = -1, off = 0;
   uint4 row_new = make_uint4(0, 0, 0, 0);
@@ -152,17 +162,24 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
 #pragma unroll
   for (int mt = 0; mt < 8; ++mt) o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f;
   const bool hv0 = 2 * t < G, hv1 = 2 * t + 1 < G;
-  float *sc = scores + (size_t)warp * p.warp_tiles * TILE * GP;
+  float *sc = (LONG ? p.scratch + (size_t)blockIdx.x * NW * p.warp_tiles * TILE * GP : scores) +
+              (size_t)warp * p.warp_tiles * TILE * GP;
+  const uint64_t acc_pol = policy_evict_last();
   int issued = min(nt, STAGES);
   int n = 0;
   for (; n < nt; ++n) {
     const uint32_t st = ring_u32 + (n % STAGES) * TILE_BYTES;
     if (!__all_sync(0xffffffffu, wait_phase(bar_u32 + (n % STAGES) * 8, (n / STAGES) & 1, p, 4, false))) break;
-    const int valid = __shfl_sync(0xffffffffu, fill, n);
+    if (LONG && n > 0 && n % 32 == 0) {
+      id = id2;
+      fill = fill2;
+      load_ids(n + 32, id2, fill2);
+    }
+    const int valid = __shfl_sync(0xffffffffu, fill, n & 31);
     if (n == n_tail) {
       const int r = off % TILE + (lane < 16 ? 0 : TILE);
       *(uint4 *)(ring + (swz<TILE>(st, r, (lane & 15) * 8) - smem_u32(ring))) = row_new;
-      store_new_token(p, b, l, kvh, p.ps, off, __shfl_sync(0xffffffffu, id, n), row_new, lane);
+      store_new_token(p, b, l, kvh, p.ps, off, __shfl_sync(0xffffffffu, id, n & 31), row_new, lane);
       __syncwarp();
     }
     /* two accumulators: half the chain of dependent MMAs */
@@ -181,8 +198,13 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
     acc[2] = (vb && hv0) ? acc[2] * p.scale_log2 : NEG_INF;
     acc[3] = (vb && hv1) ? acc[3] * p.scale_log2 : NEG_INF;
     float *srow = sc + ((size_t)n * TILE + g) * GP + 2 * t;
-    *(float2 *)srow = make_float2(acc[0], acc[1]);
-    *(float2 *)(srow + 8 * GP) = make_float2(acc[2], acc[3]);
+    if (LONG) {
+      st_v2_hint(srow, acc[0], acc[1], acc_pol);
+      st_v2_hint(srow + 8 * GP, acc[2], acc[3], acc_pol);
+    } else {
+      *(float2 *)srow = make_float2(acc[0], acc[1]);
+      *(float2 *)(srow + 8 * GP) = make_float2(acc[2], acc[3]);
+    }
     float mx0 = fmaxf(acc[0], acc[2]), mx1 = fmaxf(acc[1], acc[3]);
 #pragma unroll
     for (int x = 4; x < 32; x <<= 1) {
@@ -218,7 +240,8 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
     /* refill the stage; its reads (generic proxy) come before the copy (async) */
     __syncwarp();
     if (n + STAGES < nt) {
-      const int page = __shfl_sync(0xffffffffu, id, n + STAGES);
+      const int m = n + STAGES;
+      const int page = __shfl_sync(0xffffffffu, LONG && m / 32 != n / 32 ? id2 : id, m & 31);
       if (lane == 0) {
         fence_proxy_async_smem();
         copy_tile(n + STAGES, t0 + warp + NW * (n + STAGES), page);
@@ -365,22 +388,36 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
     }
   }
 
-  /* ---- token masses from this warp's scores, two tiles at a time ---- */
-  const uint64_t acc_pol = policy_evict_last();
-  for (int x = 0; x < nt; x += 2) {
-    const int nn = x + (lane >> 4), r = lane & 15;
-    const int page = __shfl_sync(0xffffffffu, id, min(nn, 31));
-    const int valid = __shfl_sync(0xffffffffu, fill, min(nn, 31));
-    if (nn < nt && r < valid) {
-      const float *s = sc + ((size_t)nn * TILE + r) * GP;
-      const float4 s0 = *(const float4 *)s, s1 = *(const float4 *)(s + 4);
-      const float m = token_mass(s0, s1, fm, fz);
-      const int tile = t0 + warp + NW * nn;
-      const size_t slot = (size_t)page * p.ps + (tile & (tpp - 1)) * TILE + r;
-      if (ROWS)
-        p.mass[(size_t)(l * p.Hkv + kvh) * p.slots + slot] = m;
-      else
-        red_add_u64_hint(p.mass_acc + slot, __float2ull_rn(m * MASS_SCALE), acc_pol);
+  /* ---- token masses from this warp's scores: a half warp per tile, four
+   * tiles' scores loaded before the first is used ---- */
+  if (LONG && nt > 32) load_ids(0, id, fill);
+  for (int x = 0; x < nt; x += 8) {
+    if (LONG && x > 0 && x % 32 == 0) load_ids(x, id, fill);
+    const int r = lane & 15;
+    float4 s0[4], s1[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int nn = x + 2 * k + (lane >> 4);
+      const float4 *s = (const float4 *)(sc + ((size_t)nn * TILE + r) * GP);
+      if (nn < nt) {
+        s0[k] = LONG ? __ldcg(s) : s[0];
+        s1[k] = LONG ? __ldcg(s + 1) : s[1];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int nn = x + 2 * k + (lane >> 4);
+      const int page = __shfl_sync(0xffffffffu, id, nn & 31);
+      const int valid = __shfl_sync(0xffffffffu, fill, nn & 31);
+      if (nn < nt && r < valid) {
+        const float m = token_mass(s0[k], s1[k], fm, fz);
+        const int tile = t0 + warp + NW * nn;
+        const size_t slot = (size_t)page * p.ps + (tile & (tpp - 1)) * TILE + r;
+        if (ROWS)
+          p.mass[(size_t)(l * p.Hkv + kvh) * p.slots + slot] = m;
+        else
+          red_add_u64_hint(p.mass_acc + slot, __float2ull_rn(m * MASS_SCALE), acc_pol);
+      }
     }
   }
 }
@@ -397,8 +434,11 @@ static ClusterSlots g_slots[64];   // per device ordinal; a racy first fill writ
 template <int NW>
 static cudaError_t prepare_warps(int per_sm, int *slots) {
   cudaError_t e = cudaSuccess;
-  for (const void *k : {(const void *)attn_cluster_kernel<false, true, NW>, (const void *)attn_cluster_kernel<true, false, NW>,
-                        (const void *)attn_cluster_kernel<false, false, NW>}) {
+  for (const void *k : {(const void *)attn_cluster_kernel<false, true, NW, false>,
+                        (const void *)attn_cluster_kernel<true, false, NW, false>,
+                        (const void *)attn_cluster_kernel<false, false, NW, false>,
+                        (const void *)attn_cluster_kernel<true, false, NW, true>,
+                        (const void *)attn_cluster_kernel<false, false, NW, true>}) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, CLUSTER_SMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   }
@@ -415,7 +455,7 @@ static cudaError_t prepare_warps(int per_sm, int *slots) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, attn_cluster_kernel<false, false, NW>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&n, attn_cluster_kernel<false, false, NW, false>, &cfg);
     slots[lg] = n << lg;
   }
   return e;
@@ -457,11 +497,14 @@ static int seq_tiles(const AttnBase &p, int b) {
  *     one item twice as fast (384 of 150, 76 and 99; 392 of 100, 58 and 85).
  *   More waves of clusters: launching them costs 0.0075 N (24 items of 813
  *     tiles, 30.4 and 33.9; 100 of 250, 39.6 and 43.1).
+ *   LONG, one wave: as one wave, with the score rows' way through L2 on top.  One
+ *     layer of 16 x 13,001 tokens 37.0 us, persistent 44.0; of 24 x 9,000,
+ *     37.5 and 44.9; of 50 x 4,000, 36.8 and 45.1; a step of 3 x 30,000 tokens
+ *     in 8 layers 121 and 139.  (22 shapes of 4,000 to 100,000 tokens.)
  *   Persistent: hbm and about 14 us of split, combine, ramp and tail, which a
  *     launch of several hundred us hides (2,304 items of 107 tiles: 281 us, 286
- *     with 8 warps per item).  It also takes what no cluster can: a warp has at
- *     most 32 tiles, and a CTA's scores must fit shared memory. */
-ClusterPlan cluster_plan(const AttnBase &p) {
+ *     with 8 warps per item). */
+ClusterPlan cluster_plan(const AttnBase &p, size_t scratch_floats) {
   ClusterPlan best;
   int dev = 0, T = 1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return best;
@@ -501,28 +544,50 @@ ClusterPlan cluster_plan(const AttnBase &p) {
         best.warp_tiles = n;
       }
     }
+  /* LONG: one wave only; against the persistent kernel at its measured cost
+   * for such launches, 8% of hbm above the figure that the others have to beat */
+  if (best.C == 0) least += 0.08 * hbm;
+  for (int warps = 4; warps <= 8 && (double)sum * lh * SCORE_BYTES < LONG_SCORES; warps += 4)
+    for (int lg = 0; lg < 5; ++lg) {
+      const int C = 1 << lg, n = ((T + C - 1) / C + warps - 1) / warps;
+      const long long N = items * C, slots = warps == 4 ? g_slots[dev].w4[2][lg] : g_slots[dev].w8[lg];
+      if (N > slots || (size_t)N * warps * n * TILE * GP > scratch_floats) continue;
+      const double base = warps == 4 ? (C == 1 ? 2.25 : 3.7) : (C == 1 ? 2.85 : 4.0);
+      const int shared = warps == 4 ? (int)((N - 1) / g_slots[dev].w4[0][0]) : 0;   // more CTAs on an SM
+      const double cta = (base + (warps == 4 ? 0.75 : 0.85) * n) * (1.0 + 0.1 * shared);
+      const double cost = std::max(cta, hbm + 4.0) + 0.003 * N + 1.0 + 0.1 * hbm;
+      if (cost < least) {
+        least = cost;
+        best.C = C;
+        best.warps = warps;
+        best.warp_tiles = n;
+        best.spill = true;
+      }
+    }
   return best;
 }
 
-template <int NW>
+template <int NW, bool LONG>
 static cudaError_t launch_warps(const cudaLaunchConfig_t &cfg, const ClusterParams &p, const CUtensorMap &tmap) {
-  if (!p.mass_acc) return cudaLaunchKernelEx(&cfg, attn_cluster_kernel<false, true, NW>, p, tmap);
-  return p.page_fill ? cudaLaunchKernelEx(&cfg, attn_cluster_kernel<true, false, NW>, p, tmap)
-                     : cudaLaunchKernelEx(&cfg, attn_cluster_kernel<false, false, NW>, p, tmap);
+  if (!p.mass_acc)
+    return LONG ? cudaErrorInvalidValue : cudaLaunchKernelEx(&cfg, attn_cluster_kernel<false, true, NW, false>, p, tmap);
+  return p.page_fill ? cudaLaunchKernelEx(&cfg, attn_cluster_kernel<true, false, NW, LONG>, p, tmap)
+                     : cudaLaunchKernelEx(&cfg, attn_cluster_kernel<false, false, NW, LONG>, p, tmap);
 }
 
-cudaError_t launch_cluster(const AttnBase &base, const ClusterPlan &plan, bool early, const CUtensorMap &tmap,
-                           cudaStream_t s) {
+cudaError_t launch_cluster(const AttnBase &base, const ClusterPlan &plan, bool early, float *scratch,
+                           const CUtensorMap &tmap, cudaStream_t s) {
   ClusterParams p;
   (AttnBase &)p = base;
   p.C = plan.C;
   p.warp_tiles = plan.warp_tiles;
   p.early = early;
+  p.scratch = scratch;
   p.out16 = ((uintptr_t)p.out & 15) == 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.n_seqs * p.L_launch * p.Hkv * p.C);
   cfg.blockDim = dim3(32 * plan.warps);
-  cfg.dynamicSmemBytes = cluster_smem(plan.warps, p.C, p.warp_tiles);
+  cfg.dynamicSmemBytes = cluster_smem(plan.warps, p.C, plan.spill ? 0 : p.warp_tiles);
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -533,7 +598,8 @@ cudaError_t launch_cluster(const AttnBase &base, const ClusterPlan &plan, bool e
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return plan.warps == 4 ? launch_warps<4>(cfg, p, tmap) : launch_warps<8>(cfg, p, tmap);
+  if (plan.spill) return plan.warps == 4 ? launch_warps<4, true>(cfg, p, tmap) : launch_warps<8, true>(cfg, p, tmap);
+  return plan.warps == 4 ? launch_warps<4, false>(cfg, p, tmap) : launch_warps<8, false>(cfg, p, tmap);
 }
 
 }  // namespace md

@@ -874,12 +874,12 @@ md_status run_attention(md_ctx *c, int batch, int l0, int L, int q_layers, const
   }
   /* the debug knobs of the persistent kernel's planner and exchange keep that kernel */
   const bool knobs = c->grid_cap > 0 || c->force_chunks > 0 || c->extra_arrivals > 0;
-  const ClusterPlan plan = knobs ? ClusterPlan{} : cluster_plan(base);
+  const ClusterPlan plan = knobs ? ClusterPlan{} : cluster_plan(base, (size_t)MAX_GRID * 2 * c->lay.scratch_tokens * GP);
   cudaEvent_t e0;
   cudaError_t e;
   if (plan.C > 0) {
     prof_begin(c, &e0);
-    e = launch_cluster(base, plan, k_new && l0 > 0, c->tmap_tile, c->stream);
+    e = launch_cluster(base, plan, k_new && l0 > 0, ptr<float>(c, c->lay.scratch), c->tmap_tile, c->stream);
     prof_end(c, STAGE_ATTN, e0);
     return e == cudaSuccess ? MD_OK : cuda_fail(c, e, "attention launch");
   }

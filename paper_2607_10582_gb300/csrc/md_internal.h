@@ -163,7 +163,7 @@ struct AttnParams : AttnBase {
 
 /* The cluster kernel (md_attn_cluster.cu): a cluster of C CTAs of 4 or 8
  * warps per (sequence, layer, KV head), each warp with up to 32 tiles of TILE
- * tokens. */
+ * tokens (more when the scores spill to scratch). */
 constexpr int TILE = 16;
 constexpr int MAX_CLUSTER = 16;
 struct ClusterParams : AttnBase {
@@ -171,15 +171,17 @@ struct ClusterParams : AttnBase {
   int warp_tiles;      // most tiles of any warp (sizes the score rows)
   int early;           // K/V copies may start before the kernel ahead has finished
   int out16;           // out is 16-byte aligned
+  float *scratch;      // spilled scores [CTA][warp][warp_tiles][TILE][8]
 };
 struct ClusterPlan {
   int C = 0;           // CTAs per item, or 0: the persistent kernel
   int warps = 4, warp_tiles = 0;
+  bool spill = false;  // the scores go to scratch
 };
 cudaError_t cluster_prepare();
-ClusterPlan cluster_plan(const AttnBase &p);
-cudaError_t launch_cluster(const AttnBase &p, const ClusterPlan &plan, bool early, const CUtensorMap &tmap,
-                           cudaStream_t s);
+ClusterPlan cluster_plan(const AttnBase &p, size_t scratch_floats);
+cudaError_t launch_cluster(const AttnBase &p, const ClusterPlan &plan, bool early, float *scratch,
+                           const CUtensorMap &tmap, cudaStream_t s);
 /* The tensor maps of the K/V pool (encode: the driver's cuTensorMapEncodeTiled). */
 bool encode_page_map(void *encode, CUtensorMap *m, void *pool, size_t rows, int ps);
 bool encode_tile_map(void *encode, CUtensorMap *m, void *pool, size_t rows, int ps);

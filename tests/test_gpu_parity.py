@@ -415,6 +415,9 @@ def test_entry_points_mixed_step_by_step():
     (1, 12, 2, 16, [1500 + 16 * i for i in range(12)], 0),   # clusters of CTAs of 8 warps
     (2, 16, 2, 16, [300 + 7 * i for i in range(40)], 0),     # one CTA per item, more than one wave
     (3, 5, 1, 16, [1790 - 25 * i for i in range(60)], 0),    # the same with 8 warps
+    (1, 16, 2, 32, [20000, 17, 9001], 0),                    # spilled scores, page ids in several batches
+    (2, 8, 2, 16, [6100, 4000, 5999], 1),                    # the same with region-aligned pages
+    (8, 7, 1, 16, [3500 + 50 * i for i in range(12)], 0),    # spilled scores with 4 warps
 ])
 def test_cluster_attention_follows_the_oracle(L, Hq, Hkv, ps, lengths, aligned):
     """Launch shapes that take the cluster attention kernel in each of its
