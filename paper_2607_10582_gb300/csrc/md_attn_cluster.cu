@@ -20,6 +20,8 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
+#include <mutex>
 
 #include "md_attn.cuh"
 
@@ -428,8 +430,10 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
  * take 304 CTAs of 4 warps, 288 as clusters of 8, 224 as clusters of 16). */
 struct ClusterSlots {
   int w4[3][5], w8[5];
+  std::atomic<bool> ready{false};
 };
-static ClusterSlots g_slots[64];   // per device ordinal; a racy first fill writes the same values
+static ClusterSlots g_slots[64];   // per device ordinal, filled once under g_slots_mu
+static std::mutex g_slots_mu;
 
 template <int NW>
 static cudaError_t prepare_warps(int per_sm, int *slots) {
@@ -467,11 +471,11 @@ cudaError_t cluster_prepare() {
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   ClusterSlots &g = g_slots[dev];
-  if (g.w8[0] > 0) return cudaSuccess;
-  ClusterSlots s;
-  for (int per = 3; per >= 1 && e == cudaSuccess; --per) e = prepare_warps<4>(per, s.w4[per - 1]);
-  if (e == cudaSuccess) e = prepare_warps<8>(1, s.w8);
-  if (e == cudaSuccess) g = s;
+  std::lock_guard<std::mutex> lock(g_slots_mu);
+  if (g.ready.load(std::memory_order_relaxed)) return cudaSuccess;
+  for (int per = 3; per >= 1 && e == cudaSuccess; --per) e = prepare_warps<4>(per, g.w4[per - 1]);
+  if (e == cudaSuccess) e = prepare_warps<8>(1, g.w8);
+  if (e == cudaSuccess && g.w4[0][0] > 0) g.ready.store(true, std::memory_order_release);
   return e;
 }
 
@@ -507,7 +511,9 @@ static int seq_tiles(const AttnBase &p, int b) {
 ClusterPlan cluster_plan(const AttnBase &p, size_t scratch_floats) {
   ClusterPlan best;
   int dev = 0, T = 1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return best;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 ||
+      !g_slots[dev].ready.load(std::memory_order_acquire))
+    return best;
   long long sum = 0;
   for (int b = 0; b < p.n_seqs; ++b) {
     const int t = seq_tiles(p, b);

@@ -26,6 +26,7 @@ using namespace md;
 
 namespace {
 
+constexpr size_t COPY_KERNEL_BYTES = (size_t)16 << 20;   // md_get_state: most bytes copied by a kernel
 constexpr int N_STAGES = 5;
 constexpr int STAGE_APPEND = 0, STAGE_ATTN = 1, STAGE_FOLD = 2, STAGE_SCORE = 3,
               STAGE_SELECT = 4;
@@ -74,6 +75,7 @@ struct md_ctx {
   int plan_batch = -1, plan_layers = -1, plan_T = 0, plan_G = 0;
   int plan_knobs[5] = {-1, -1, -1, -1, -1};
   bool calib_on = false;     // calibration histogram being gathered
+  int device = 0;
   int pageable_access = 0;   // the device reads and writes pageable host memory coherently
   int zero_copy = 1;         // md_decode_step_host: new K/V and output used in place when reachable
   bool prof = false;
@@ -570,6 +572,7 @@ MD_API md_status md_create(const md_config *cfg, md_ctx **out) {
   }
   {
     int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) c->device = dev;
     if (cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&v, cudaDevAttrPageableMemoryAccess, dev) == cudaSuccess)
       c->pageable_access = v;
@@ -1229,7 +1232,15 @@ MD_API md_status md_get_state(md_ctx *c, int what, void *dst, size_t bytes) {
   size_t off, n;
   if (!state_array(c, what, &off, &n)) return fail(c, MD_ERR_INVALID_ARG, "unknown state array");
   if (bytes != n) return fail(c, MD_ERR_INVALID_ARG, "state array is %zu bytes, not %zu", n, bytes);
-  cudaError_t e = cudaMemcpyAsync(dst, c->ws + off, n, cudaMemcpyDeviceToDevice, c->stream);
+  /* by a kernel where dst is this device's memory and aligned for it; the
+   * K/V pool and other large arrays are left to the copy engine */
+  cudaPointerAttributes at;
+  cudaError_t e;
+  if (n <= COPY_KERNEL_BYTES && n % 16 == 0 && ((uintptr_t)dst & 15) == 0 &&
+      cudaPointerGetAttributes(&at, dst) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == c->device)
+    e = launch_copy({(const uint4 *)(c->ws + off), (uint4 *)dst, n / 16}, c->stream);
+  else
+    e = cudaMemcpyAsync(dst, c->ws + off, n, cudaMemcpyDeviceToDevice, c->stream);
   return e == cudaSuccess ? MD_OK : cuda_fail(c, e, "state copy");
 }
 

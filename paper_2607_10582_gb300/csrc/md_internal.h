@@ -49,6 +49,14 @@ struct Layout {
 
 size_t compute_layout(const md_config &c, Layout *lay);
 
+/* --------------------------------------------------------- state copy --- */
+struct CopyParams {
+  const uint4 *src;
+  uint4 *dst;
+  size_t n;                              // 16-byte pieces, at least 1
+};
+cudaError_t launch_copy(const CopyParams &p, cudaStream_t s);
+
 /* ------------------------------------------------------------- append --- */
 /* The arrays an append writes. */
 struct AppendTo {

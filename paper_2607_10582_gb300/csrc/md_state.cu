@@ -43,6 +43,23 @@ cudaError_t launch_init(int32_t *free_stack, int P_phys, int *status, int *count
   return cudaGetLastError();
 }
 
+/* ---------------------------------------------------------- state copy --- */
+/* Device-to-device copy of a state array, 16 bytes per thread and iteration.
+ * In a stream of dependent launches it starts as the kernel ahead ends, where
+ * a copy node waits for that one and holds up the next: a pass over 32
+ * sequences of 430 tokens that reads four arrays back, 97.9 -> 87.9 us. */
+__global__ void __launch_bounds__(256) copy_kernel(const __grid_constant__ CopyParams p) {
+  pdl_wait();
+  pdl_trigger();
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < p.n; i += (size_t)gridDim.x * blockDim.x)
+    p.dst[i] = p.src[i];
+}
+
+cudaError_t launch_copy(const CopyParams &p, cudaStream_t s) {
+  const size_t blocks = (p.n + 255) / 256;
+  return launch_pdl(copy_kernel, (int)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, s, p);
+}
+
 /* -------------------------------------------------------------- append --- */
 __device__ __forceinline__ void start_token(const AppendTo &d, size_t slot, int region, int step) {
   d.region[slot] = (uint8_t)region;

@@ -630,6 +630,24 @@ def test_argument_forms_give_the_same_step():
         assert torch.equal(reg, seen[0][1]) and torch.equal(tab, seen[0][2])
 
 
+@pytest.mark.parametrize("pages", [1, 3, 4097])
+def test_state_copies_at_any_address(pages):
+    """Every state array reads back the same into an aligned buffer (copied by
+    a kernel where it is small) and into one that is not aligned for that."""
+    c = md.Cache(1, 4, 1, 16, 2, pages, pages)
+    k, v = synth.kv_host(29, 0, 1, 1, 0, 16)
+    c.append_tokens(1, np.arange(16) % 7, to_dev(k), to_dev(v), -np.arange(16))
+    for what in range(15):
+        a = c.get_state(what)
+        raw = a.contiguous().view(torch.uint8).view(-1)
+        buf = torch.zeros(raw.numel() + 32, dtype=torch.uint8, device="cuda")
+        off = 1 if a.element_size() == 1 else a.element_size()
+        assert md.lib().md_get_state(c.h, what, buf.data_ptr() + off, raw.numel()) == md.MD_OK
+        assert torch.equal(buf[off:off + raw.numel()], raw), what
+        assert int(buf[:off].sum()) == 0 and int(buf[off + raw.numel():].sum()) == 0, what
+    c.close()
+
+
 def test_checkpoint_restore_replays_step():
     w = synth.custom_workload("ckpt", L=2, Hq=8, Hkv=2, page_size=16, lengths=[900],
                               budget_frac=0.3, steps=2, seed=9)
