@@ -217,7 +217,7 @@ struct CalibSmem {
  * A token's step mass is one fixed-point accumulator (the attention kernel
  * adds every (layer, KV head) into it): read and zeroed here, loaded together
  * with the token's state. */
-template <int PS>
+template <int PS, bool CALIB>
 __device__ __forceinline__ float score_tile(const ScoreParams &p, int b, int pg, int off, bool page_ok, bool need_mass,
                                             CalibSmem *calib) {
   const float INF = INFINITY;
@@ -241,14 +241,15 @@ __device__ __forceinline__ float score_tile(const ScoreParams &p, int b, int pg,
       tr = p.t_ref[slot];
       if (p.observe) w = p.window[slot];
       if (p.observe || p.score_mode == 2) ntok = p.seq_tokens ? p.seq_tokens[b] : p.n_tokens[b];
-      if (calib || p.score_mode == 3) tins = p.t_ins[slot];
+      if (CALIB || p.score_mode == 3) tins = p.t_ins[slot];
     }
   }
   /* the sum over layers and query heads, rounded once to fp32 */
   const float msum = __ull2float_rn(macc) * MASS_UNIT;
   if (valid && need_mass) p.mass_acc[slot] = 0ull;
   float s = 0.f;
-  int pinned = 0;
+  int pinned = 0, bin = -1;
+  unsigned long long fx = 0ull;
   if (valid) {
     if (p.fold_only) {
       p.window[slot] = w + msum;
@@ -263,12 +264,12 @@ __device__ __forceinline__ float score_tile(const ScoreParams &p, int b, int pg,
         p.ahat[slot] = abar;
         p.a[slot] = a;
         p.t_ref[slot] = tr;
-        if (calib) {
+        if (CALIB) {
           const int age = p.t - tins;
           const int bkt = age >= 0 ? age / CALIB_WIDTH : -1;
           if (bkt >= 0 && bkt < CALIB_BUCKETS) {
-            atomicAdd(&calib->sum[reg * CALIB_BUCKETS + bkt], __float2ull_rn(abar * 4294967296.0f));
-            atomicAdd(&calib->cnt[reg * CALIB_BUCKETS + bkt], 1u);
+            bin = reg * CALIB_BUCKETS + bkt;
+            fx = __float2ull_rn(abar * 4294967296.0f);
           }
         }
       }
@@ -287,6 +288,35 @@ __device__ __forceinline__ float score_tile(const ScoreParams &p, int b, int pg,
     }
   }
   if (p.fold_only) return 0.f;
+  if (CALIB) {
+    /* one pair of shared atomics for all tokens of a bin that holds a quarter
+     * of the warp's (a prompt's page has one or two bins) instead of one pair
+     * per token: the histogram's share of an observation of 16 x 30,000 tokens,
+     * 30 -> 3 us; of 12 x 2,400, 12 -> 4 us.  Tokens spread over more bins (a
+     * page of decode steps: four to a bin) conflict less and go one by one. */
+    unsigned left = __ballot_sync(0xffffffffu, bin >= 0);
+    while (left) {
+      const int first = __ffs(left) - 1, cur = __shfl_sync(0xffffffffu, bin, first);
+      const unsigned in = __ballot_sync(0xffffffffu, bin == cur);
+      if (__popc(in) < 8) {
+        if ((left >> (threadIdx.x & 31)) & 1) {
+          atomicAdd(&calib->sum[bin], fx);
+          atomicAdd(&calib->cnt[bin], 1u);
+        }
+        break;
+      }
+      const unsigned long long v = bin == cur ? fx : 0ull;
+      const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)v & 0xFFFFFFu);
+      const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 24) & 0xFFFFFFu);
+      const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 48));
+      if ((threadIdx.x & 31) == first) {
+        atomicAdd(&calib->sum[cur], (unsigned long long)lo + ((unsigned long long)mid << 24) + ((unsigned long long)hi << 48));
+        atomicAdd(&calib->cnt[cur], (unsigned)__popc(in));
+      }
+      left &= ~in;
+    }
+    __syncwarp();
+  }
   float sum = (valid && !pinned) ? s : 0.f;
   float mx = (valid && !pinned) ? s : -INF;
   int anyp = (valid && pinned) ? 1 : 0;
@@ -308,21 +338,21 @@ __device__ __forceinline__ float score_tile(const ScoreParams &p, int b, int pg,
 /* One warp per tile; the loop count is uniform across a warp, so the segmented
  * shuffle reductions see every lane.  The launcher sizes the grid to one wave
  * of resident blocks. */
-template <int PS>
+template <int PS, bool CALIB>
 __global__ void __launch_bounds__(256, 6) score_kernel(const __grid_constant__ ScoreParams p) {
   pdl_wait();
   pdl_trigger();
   constexpr int PPW = 32 / PS;
-  __shared__ CalibSmem hist;
+  __shared__ __align__(8) uint8_t hist_mem[CALIB ? sizeof(CalibSmem) : 8];
+  CalibSmem *hist = (CalibSmem *)hist_mem;
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   const int tiles = (p.total_pages + PPW - 1) / PPW;
   const bool need_mass = p.fold_only || (p.observe && p.mass_pending);
-  const bool calib = p.calib_on && p.observe && !p.fold_only;
-  if (calib) {
+  if (CALIB) {
     for (int k = threadIdx.x; k < 8 * CALIB_BUCKETS; k += blockDim.x) {
-      hist.sum[k] = 0ull;
-      hist.cnt[k] = 0u;
+      hist->sum[k] = 0ull;
+      hist->cnt[k] = 0u;
     }
     __syncthreads();
   }
@@ -330,14 +360,14 @@ __global__ void __launch_bounds__(256, 6) score_kernel(const __grid_constant__ S
     const int gp = (t0 + wib) * PPW + lane / PS;
     const bool page_ok = gp < p.total_pages;
     const int b = page_ok ? find_seq(p.page_start, p.n_seqs, gp) : 0;
-    score_tile<PS>(p, b, page_ok ? gp - p.page_start[b] : 0, lane % PS, page_ok, need_mass, calib ? &hist : nullptr);
+    score_tile<PS, CALIB>(p, b, page_ok ? gp - p.page_start[b] : 0, lane % PS, page_ok, need_mass, hist);
   }
-  if (calib) {
+  if (CALIB) {
     __syncthreads();
     for (int k = threadIdx.x; k < 8 * CALIB_BUCKETS; k += blockDim.x)
-      if (hist.cnt[k]) {
-        atomicAdd(&p.calib_sum[k], hist.sum[k]);
-        atomicAdd(&p.calib_cnt[k], hist.cnt[k]);
+      if (hist->cnt[k]) {
+        atomicAdd(&p.calib_sum[k], hist->sum[k]);
+        atomicAdd(&p.calib_cnt[k], hist->cnt[k]);
       }
   }
 }
@@ -346,7 +376,7 @@ __global__ void __launch_bounds__(256, 6) score_kernel(const __grid_constant__ S
  * (SMs x blocks per SM from the occupancy of the instance).  The kernel gives
  * every block an equal share of the pages, so a grid larger than one wave
  * would leave the second wave's blocks as a tail. */
-template <int PS>
+template <int PS, bool CALIB>
 static int score_grid_cap() {
   static int cached[64];   // per device ordinal; a racy first fill writes the same value
   int dev = 0;
@@ -354,21 +384,25 @@ static int score_grid_cap() {
   if (cached[dev] > 0) return cached[dev];
   int sms = 0, per_sm = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, score_kernel<PS>, 256, 0) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, score_kernel<PS, CALIB>, 256, 0) != cudaSuccess ||
       sms <= 0 || per_sm <= 0)
     return 152 * 4;
   cached[dev] = sms * per_sm;
   return cached[dev];
 }
 
+template <int PS, bool CALIB>
+static cudaError_t launch_score_ps(const ScoreParams &p, cudaStream_t s) {
+  const int ppb = 256 / PS;   // pages per block and iteration: one warp per tile
+  const long long blocks = (p.total_pages + ppb - 1) / ppb, cap = score_grid_cap<PS, CALIB>();
+  return launch_pdl(score_kernel<PS, CALIB>, (int)(blocks < cap ? blocks : cap), 256, 0, s, p);
+}
+
 cudaError_t launch_score(const ScoreParams &p, cudaStream_t s) {
   if (p.total_pages == 0) return cudaSuccess;
-  const int ppb = 256 / p.ps;   // pages per block and iteration: one warp per tile
-  const int cap = p.ps == 16 ? score_grid_cap<16>() : score_grid_cap<32>();
-  long long blocks = (p.total_pages + ppb - 1) / ppb;
-  if (blocks > cap) blocks = cap;
-  if (p.ps == 16) return launch_pdl(score_kernel<16>, (int)blocks, 256, 0, s, p);
-  return launch_pdl(score_kernel<32>, (int)blocks, 256, 0, s, p);
+  if (p.calib_on && p.observe && !p.fold_only)
+    return p.ps == 16 ? launch_score_ps<16, true>(p, s) : launch_score_ps<32, true>(p, s);
+  return p.ps == 16 ? launch_score_ps<16, false>(p, s) : launch_score_ps<32, false>(p, s);
 }
 
 /* -------------------------------------------------------------- select --- */
@@ -577,7 +611,7 @@ __global__ void __launch_bounds__(1024) observe_kernel(const __grid_constant__ O
   if (tid < OBSERVE_PAGES && tid >= P) keys[tid] = KEY_PINNED;
   for (int pg0 = warp * PPW; pg0 < P; pg0 += (int)(blockDim.x >> 5) * PPW) {
     const int pg = pg0 + lane / PS;
-    const float S = score_tile<PS>(p.s, b, pg < P ? pg : 0, lane % PS, pg < P, p.s.observe && p.s.mass_pending, nullptr);
+    const float S = score_tile<PS, false>(p.s, b, pg < P ? pg : 0, lane % PS, pg < P, p.s.observe && p.s.mass_pending, nullptr);
     if (pg < P && lane % PS == 0) keys[pg] = S == INFINITY ? KEY_PINNED : order_key(S);
   }
   __syncthreads();
