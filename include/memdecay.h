@@ -166,7 +166,8 @@ md_status md_decode_step(md_ctx *ctx, int batch, const void *q_dev, const void *
                          const void *v_new_dev, const uint8_t *new_region_host, void *out_dev);
 
 /* md_decode_step with the step's tensors in host memory.  The query rows
- * are copied into the workspace before the step.  The new tokens' K/V and
+ * are copied into the workspace before the step (by the append kernel where
+ * they are pinned).  The new tokens' K/V and
  * the output are used where they are when the device can reach them: the
  * kernels read the K/V rows and write the output over the host link (on a
  * GB300, NVLink-C2C), with no copy.  The device reaches pinned (page-locked)
@@ -288,7 +289,9 @@ md_status md_load_state(md_ctx *ctx, const void *src_dev, const void *host_blob)
 
 /* Per-stage GPU time, from CUDA events recorded around each launch while
  * enabled.  Stages: 0 append, 1 attention (stage 1), 2 window fold,
- * 3 score + page reduce (stages 2-3), 4 select + compact (stage 4).
+ * 3 score + page reduce (stages 2-3), 4 select + compact (stage 4).  Decode
+ * steps with device buffers append inside the attention launch (counted there),
+ * and short sequences are scored and selected in one launch (counted as 3).
  * md_profile_read synchronises the stream and returns, for each stage, the
  * summed milliseconds and the number of launches since enabling.  Each event
  * pair keeps consecutive kernels from overlapping (about 2 us per event on a
@@ -298,7 +301,8 @@ md_status md_profile_enable(md_ctx *ctx, int enable);
 md_status md_profile_read(md_ctx *ctx, double *ms_per_stage, int64_t *launches_per_stage,
                           int n_stages);
 
-/* Test and tuning support.
+/* Test and tuning support.  GRID_LIMIT, FORCE_CHUNKS and EXTRA_ARRIVALS keep
+ * the persistent attention kernel, which they are about.
  *   MD_DEBUG_SPIN_LIMIT_NS    limit of each device-side wait (default 2e9)
  *   MD_DEBUG_EXTRA_ARRIVALS   extra arrivals the attention exchange waits for
  *                             on its next launch (a wait nothing completes;
@@ -378,6 +382,7 @@ md_status md_calib_fit(const double *mass_sum, const int64_t *count, int n_bucke
  * The kernel's scratch memory (score rows, split partials, arrival counters,
  * status words) lives in one fixed 24 MiB device array inside the library,
  * which every GPU that loads the library holds until the process exits.
+ * Small launches take the cluster kernel, which needs none of it.
  * Nothing is allocated by this call.
  *
  *   kv_pool_dev      bf16 [L][num_phys_pages][Hkv][2][page_size][128]: for

@@ -542,12 +542,11 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
     fence_barrier_init();
   }
   __syncthreads();
-  /* The kernel ahead in the stream (the step's append) writes the new
-   * token's K/V into each sequence's last page, that page's block-table
-   * entry and fill, and the new token's state.  Every thread waits for it
-   * before its first global access, except the producer's issuing lane,
-   * which first starts its first unit's copies that append cannot touch
-   * (the query rows and the pages before the sequence's last one). */
+  /* The kernel ahead in the stream may still be writing the block table, the
+   * pool or (a step with host buffers) the query rows: every thread waits for
+   * it before its first global access.  Only the no-allocation call, whose
+   * cache nothing of this library writes, lets the producer's issuing lane
+   * start its first unit's copies before. */
   const bool issuer = warp == 0 && lane == 0;
   if (!issuer) {
     pdl_wait();
@@ -578,7 +577,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
         un = decode_unit(p, u);
         pb = un.p0;
       }
-      if (u < p.total_units && !NEW) {
+      if (u < p.total_units && ROWS) {
         /* before the wait: the first unit's query rows (the caller's) and,
          * when the unit is its item's only chunk, its pages below the
          * sequence's last one, at most one per stage (measured on a GB300:
@@ -621,7 +620,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
           }
         }
         if (nxu < p.total_units) cntn = load_batch<ALIGNED, NEW>(p, nx, npb, nx.p1, phn, fln);
-        if (pb == un.p0 && (NEW || u != (int)blockIdx.x)) {   // not NEW: the first unit's went out before the wait
+        if (pb == un.p0 && (!ROWS || u != (int)blockIdx.x)) {   // ROWS: the first unit's went out before the wait
           /* the unit's G query rows (and the new token's K and V rows, where
            * the unit holds its page) into a double-buffered slot */
           const int qs = nu & 1;

@@ -797,13 +797,18 @@ md_status begin_step(md_ctx *c, int batch, const uint8_t *new_region_host) {
 
 /* The step's append as a launch of its own, for new K/V that lie in host
  * memory: every layer's rows in one pass over the host link, where the
- * attention units' reads of two short rows each would pay its latency. */
-md_status append_step(md_ctx *c, int batch, const void *k_new, const void *v_new) {
+ * attention units' reads of two short rows each would pay its latency.  With
+ * q_src (pinned host memory) the pass brings the query rows as well. */
+md_status append_step(md_ctx *c, int batch, const void *k_new, const void *v_new, const void *q_src, void *q_dst,
+                      size_t q_bytes) {
   const md_config &cf = c->cfg;
   AppendStepParams ap;
   ap.to = append_to(c);
   ap.k_src = (const uint16_t *)k_new;
   ap.v_src = (const uint16_t *)v_new;
+  ap.q_src = (const uint4 *)q_src;
+  ap.q_dst = (uint4 *)q_dst;
+  ap.q_n = q_src ? (unsigned)(q_bytes / 16) : 0;
   ap.n_seqs = batch;
   ap.insert_step = (int)c->m.t;
   for (int b = 0; b < batch; ++b) {
@@ -921,7 +926,7 @@ namespace {
  * host memory only where the device accesses pageable memory coherently
  * (Grace's NVLink-C2C with address translation).  16-byte alignment is
  * required (the kernels move 16-byte pieces). */
-void *device_view(const md_ctx *c, const void *h) {
+void *device_view(const md_ctx *c, const void *h, bool pinned_only = false) {
   if ((uintptr_t)h & 15) return nullptr;
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, h) != cudaSuccess) {
@@ -929,7 +934,7 @@ void *device_view(const md_ctx *c, const void *h) {
     return nullptr;
   }
   if (a.type == cudaMemoryTypeHost && a.devicePointer) return ((uintptr_t)a.devicePointer & 15) ? nullptr : a.devicePointer;
-  if (a.type == cudaMemoryTypeUnregistered && c->pageable_access) return const_cast<void *>(h);
+  if (a.type == cudaMemoryTypeUnregistered && c->pageable_access && !pinned_only) return const_cast<void *>(h);
   return nullptr;
 }
 
@@ -970,22 +975,25 @@ MD_API md_status md_decode_step_host(md_ctx *c, int batch, const void *q_host, c
    * device can reach them: the append kernel reads the K/V rows and the
    * attention kernel writes the output over the host link, with no copy (on
    * a GB300 that took the config-2 steady step's device time from 170 to
-   * 138 us).  The query rows are always copied into the workspace first:
-   * every unit of the attention kernel reads its rows with a TMA copy at its
-   * start, and over the host link that latency cost more than the copy
-   * (207 us).  Buffers the device cannot reach are copied too. */
+   * 138 us).  The query rows are always copied into the workspace first, by
+   * the append kernel where they are pinned: every unit of the attention
+   * kernel reads its rows at its start, and over the host link that latency
+   * cost more than the copy (207 us).  Buffers the device cannot reach are
+   * copied too. */
   const void *vk = c->zero_copy ? device_view(c, k_new_host) : nullptr;
   const void *vv = c->zero_copy ? device_view(c, v_new_host) : nullptr;
+  const void *vq = c->zero_copy ? device_view(c, q_host, true) : nullptr;
   void *vo = c->zero_copy ? device_view(c, out_host) : nullptr;
   uint8_t *dq = c->ws + c->lay.io_q, *dk = c->ws + c->lay.io_k, *dv = c->ws + c->lay.io_v,
           *dout = c->ws + c->lay.io_out;
-  cudaError_t e = cudaMemcpyAsync(dq, q_host, q_bytes, cudaMemcpyHostToDevice, c->stream);
+  cudaError_t e = cudaSuccess;
+  if (!vq) e = cudaMemcpyAsync(dq, q_host, q_bytes, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess && !vk) e = cudaMemcpyAsync(dk, k_new_host, kv_bytes, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess && !vv) e = cudaMemcpyAsync(dv, v_new_host, kv_bytes, cudaMemcpyHostToDevice, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "input copy");
   st = begin_step(c, batch, new_region_host);
   if (st != MD_OK) return st;
-  st = append_step(c, batch, vk ? vk : dk, vv ? vv : dv);
+  st = append_step(c, batch, vk ? vk : dk, vv ? vv : dv, vq, dq, q_bytes);
   if (st != MD_OK) return st;
   st = run_attention(c, batch, 0, cf.num_layers, cf.num_layers, dq, nullptr, nullptr, vo ? vo : dout);
   if (st != MD_OK) return st;

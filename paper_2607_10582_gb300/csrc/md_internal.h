@@ -75,6 +75,9 @@ struct AppendTo {
 struct AppendStepParams {
   AppendTo to;
   const uint16_t *k_src, *v_src;
+  const uint4 *q_src;                    // query rows to bring into the workspace on the way
+  uint4 *q_dst;
+  unsigned q_n;                          // their 16-byte pieces, or 0
   int n_seqs, insert_step;
   int tok0[MD_MAX_BATCH];                // slot of the token in its sequence
   int pop[MD_MAX_BATCH];                 // free-stack index of the page it opens, or -1
