@@ -72,11 +72,11 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
   const int G = p.G, C = p.C;
   const float NEG_INF = -INFINITY;
 
-  if (lane < STAGES) mbar_init(bar_u32 + lane * 8, 1);
-  if (lane == 0) {
+  if (lane < STAGES) {   // each barrier is made visible by the lane that initialised it
+    mbar_init(bar_u32 + lane * 8, 1);
     fence_barrier_init();
-    tma_prefetch_desc(&tmap);
   }
+  if (lane == 0) tma_prefetch_desc(&tmap);
   __syncwarp();
   if (C > 1) cluster_arrive();   // this CTA runs: the others may write its shared memory
 
