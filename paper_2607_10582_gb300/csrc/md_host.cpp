@@ -1242,10 +1242,15 @@ MD_API md_status md_get_state(md_ctx *c, int what, void *dst, size_t bytes) {
   if (bytes != n) return fail(c, MD_ERR_INVALID_ARG, "state array is %zu bytes, not %zu", n, bytes);
   /* by a kernel where dst is this device's memory and aligned for it; the
    * K/V pool and other large arrays are left to the copy engine */
-  cudaPointerAttributes at;
+  bool here = n <= COPY_KERNEL_BYTES && n % 16 == 0 && ((uintptr_t)dst & 15) == 0;
+  if (here) {
+    cudaPointerAttributes at;
+    here = cudaPointerGetAttributes(&at, dst) == cudaSuccess;
+    if (!here) cudaGetLastError();
+    here = here && at.type == cudaMemoryTypeDevice && at.device == c->device;
+  }
   cudaError_t e;
-  if (n <= COPY_KERNEL_BYTES && n % 16 == 0 && ((uintptr_t)dst & 15) == 0 &&
-      cudaPointerGetAttributes(&at, dst) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == c->device)
+  if (here)
     e = launch_copy({(const uint4 *)(c->ws + off), (uint4 *)dst, n / 16}, c->stream);
   else
     e = cudaMemcpyAsync(dst, c->ws + off, n, cudaMemcpyDeviceToDevice, c->stream);
