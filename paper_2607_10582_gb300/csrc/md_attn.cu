@@ -88,7 +88,8 @@ struct AttnShape {
   static constexpr int MERGE_FLOATS = NCW * (24 + GP * D);
   static constexpr int FIN_FLOATS = 16 + 3 * MD_MAX_CHUNKS * GP;
   static constexpr int OBUF_FLOATS = GP * D + MD_MAX_CHUNKS;   // C slices of ceil(G*D/C)
-  static constexpr size_t SMEM = 1024 + RING_BYTES + 2 * Q_BYTES + (2 * R + 10) * 8 +
+  static constexpr int ZERO_BYTES = 128;             // a row of zeros in place of stale V rows
+  static constexpr size_t SMEM = 1024 + RING_BYTES + 2 * Q_BYTES + ZERO_BYTES + (2 * R + 10) * 8 +
                                  4 * MERGE_FLOATS + 4 * FIN_FLOATS + 8 * MAX_UNIT_PAGES +
                                  4 * OBUF_FLOATS + 4 * R + 64;
 };
@@ -499,7 +500,8 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *ring = smem;
   uint8_t *sQ = ring + S::RING_BYTES;                   // [2][8 heads][128] bf16
-  uint64_t *full = (uint64_t *)(sQ + 2 * S::Q_BYTES);
+  uint4 *zero_row = (uint4 *)(sQ + 2 * S::Q_BYTES);
+  uint64_t *full = (uint64_t *)(zero_row + S::ZERO_BYTES / 16);
   uint64_t *empty = full + S::R;
   uint64_t *qfull = empty + S::R;                       // [2]
   uint64_t *qempty = qfull + 2;                         // [2]
@@ -524,8 +526,10 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
   const int lane = threadIdx.x & 31;
   const uint32_t ring_u32 = smem_u32(ring);
   const uint32_t sQ_u32 = smem_u32(sQ);
+  const uint32_t zero_u32 = smem_u32(zero_row);
   const int G = p.G;
 
+  if (threadIdx.x < S::ZERO_BYTES / 16) zero_row[threadIdx.x] = make_uint4(0, 0, 0, 0);
   if (threadIdx.x == 0) {
     for (int s = 0; s < S::R; ++s) {
       mbar_init(smem_u32(&full[s]), 1);
@@ -842,11 +846,11 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
         l1 += p01 + p11;
         const uint32_t b0 = movmatrix_trans(pack_bf16(p00, p01));
         const uint32_t b1 = movmatrix_trans(pack_bf16(p10, p11));
+        const VRow vr = v_row<PS>(st, zero_u32, tt * 16 + (mi >> 1) * 8 + rr, fill);
 #pragma unroll
         for (int mt = 0; mt < 8; ++mt) {
           uint32_t a0, a1, a2, a3;
-          ldmatrix_x4_trans(swz<PS>(st, PS + tt * 16 + (mi >> 1) * 8 + rr, mt * 16 + (mi & 1) * 8),
-                            a0, a1, a2, a3);
+          ldmatrix_x4_trans(v_chunk(vr, rr, mt * 16 + (mi & 1) * 8), a0, a1, a2, a3);
           mma_bf16(o[mt], a0, a1, a2, a3, b0, b1);
         }
       }

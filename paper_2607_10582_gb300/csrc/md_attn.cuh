@@ -47,6 +47,28 @@ __device__ __forceinline__ uint32_t swz(uint32_t stage, int row, int d) {
   return stage + half * (2 * PS * 128) + row * 128 + ((chunk ^ (row & 7)) << 4);
 }
 
+/* The V row that a lane's ldmatrix reads (row PS + v of a stage), as the row's
+ * address in either 64-column half: the stage's while token v is one of its
+ * `valid` cached tokens, else a row of zeros.  A masked token's weight is 0,
+ * but the MMA would multiply it with whatever its slot holds, and 0 times a
+ * stale Inf or NaN (an uninitialised row of a caller's pool, a page another
+ * sequence left) is NaN in every head's output.  Choosing the address costs a
+ * few instructions per tile; zeroing the stale rows in the stage, in code that
+ * only a partial tile runs, took 0.25 to 0.4 us of a 6.4 us layer launch (a
+ * cold branch), masking the fragments 0.16. */
+struct VRow {
+  uint32_t half0, half1;
+};
+template <int PS>
+__device__ __forceinline__ VRow v_row(uint32_t stage, uint32_t zero_row, int v, int valid) {
+  const uint32_t row = stage + (PS + v) * 128;
+  return {v < valid ? row : zero_row, v < valid ? row + 2 * PS * 128 : zero_row};
+}
+/* Address of the 16-byte chunk holding dims d .. d+7 of such a row. */
+__device__ __forceinline__ uint32_t v_chunk(const VRow &r, int v, int d) {
+  return (d < 64 ? r.half0 : r.half1) + ((((d & 63) >> 3) ^ (v & 7)) << 4);
+}
+
 /* A decode step's new token: one warp writes the K and V rows (16 bytes per
  * lane: K in lanes 0..15, V in 16..31) to token `off` of page `phys`; lane 0
  * of the first layer's KV head 0 starts the token's state. */

@@ -34,8 +34,9 @@ constexpr int HALF_BYTES = TILE_BYTES / 2;        // their 64-column halves
 constexpr int OS = D + 4;                         // padded row of a warp's O^T (conflict-free stores)
 constexpr int SCORE_BYTES = TILE * GP * 4;        // one tile's raw scores
 constexpr int STAGES = 2;                         // tiles in flight per warp
-/* barriers, wm, wl [warps][8], fin [16] */
-constexpr int misc_bytes(int warps) { return warps * STAGES * 8 + (2 * warps * GP + 2 * GP) * 4; }
+constexpr int ZERO_BYTES = 128;                   // a row of zeros in place of stale V rows
+/* zeros, barriers, wm, wl [warps][8], fin [16] */
+constexpr int misc_bytes(int warps) { return ZERO_BYTES + warps * STAGES * 8 + (2 * warps * GP + 2 * GP) * 4; }
 /* from every CTA of the cluster: (m, Z) per head, its O over this CTA's slice */
 constexpr int XCH_BYTES = (MAX_CLUSTER * GP * 2 + GP * D) * 4;
 constexpr int CLUSTER_SMEM = 227 * 1024, SM_SMEM = 228 * 1024;   // most a block may have, an SM has
@@ -57,7 +58,8 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
   extern __shared__ uint8_t smem_raw[];
   uint8_t *ring = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   float *scores = (float *)(ring + NW * STAGES * TILE_BYTES);
-  float *wm = scores + (LONG ? 0 : (size_t)NW * p.warp_tiles * TILE * GP);
+  float *zero_row = scores + (LONG ? 0 : (size_t)NW * p.warp_tiles * TILE * GP);
+  float *wm = zero_row + ZERO_BYTES / 4;
   float *wl = wm + NW * GP;
   float *fin = wl + NW * GP;      // [16] the item's per-head max, then 1/Z (one chunk per item)
   uint64_t *full = (uint64_t *)(fin + 2 * GP);
@@ -69,6 +71,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
   const int mi = lane >> 3, rr = lane & 7;
   const uint32_t ring_u32 = smem_u32(ring) + warp * STAGES * TILE_BYTES;   // this warp's stages
   const uint32_t bar_u32 = smem_u32(full + warp * STAGES);
+  const uint32_t zero_u32 = smem_u32(zero_row);
   const int G = p.G, C = p.C;
   const float NEG_INF = -INFINITY;
 
@@ -77,6 +80,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
     fence_barrier_init();
   }
   if (lane == 0) tma_prefetch_desc(&tmap);
+  if (lane < ZERO_BYTES / 16) ((uint4 *)zero_row)[lane] = make_uint4(0, 0, 0, 0);   // every warp: all write the same
   __syncwarp();
   if (C > 1) cluster_arrive();   // this CTA runs: the others may write its shared memory
 
@@ -233,10 +237,11 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
     l1 += p01 + p11;
     const uint32_t b0 = movmatrix_trans(pack_bf16(p00, p01));
     const uint32_t b1 = movmatrix_trans(pack_bf16(p10, p11));
+    const VRow vr = v_row<TILE>(st, zero_u32, (mi >> 1) * 8 + rr, valid);
 #pragma unroll
     for (int mt = 0; mt < 8; ++mt) {
       uint32_t a0, a1, a2, a3;
-      ldmatrix_x4_trans(swz<TILE>(st, TILE + (mi >> 1) * 8 + rr, mt * 16 + (mi & 1) * 8), a0, a1, a2, a3);
+      ldmatrix_x4_trans(v_chunk(vr, rr, mt * 16 + (mi & 1) * 8), a0, a1, a2, a3);
       mma_bf16(o[mt], a0, a1, a2, a3, b0, b1);
     }
     /* refill the stage; its reads (generic proxy) come before the copy (async) */

@@ -584,6 +584,47 @@ def test_append_inside_attention_writes_what_the_append_kernel_writes(ps, aligne
         c.close()
 
 
+@pytest.mark.parametrize("ps,aligned,persistent", [(16, 0, 0), (32, 0, 0), (32, 1, 0), (16, 0, 1), (32, 0, 1),
+                                                   (16, 1, 1), (32, 1, 1)])
+@pytest.mark.parametrize("entry", ["device", "host"])
+def test_recycled_pages_leave_nothing_in_the_output(ps, aligned, persistent, entry):
+    """Pages that an evicted sequence with infinite and NaN values leaves behind
+    give the next sequence the same output and masses, bit for bit, as pages
+    never used: what a slot past a page's tokens holds must not reach them."""
+    L, Hq, Hkv, n = 2, 16, 2, 3 * 101 + 1
+    lab = (np.arange(n) // 101 % 7).astype(np.uint8)       # aligned: partly filled pages inside
+    k, v = (to_dev(x) for x in synth.kv_host(37, 0, L, Hkv, 0, n, lab))
+    bad = torch.full_like(v, 0x7F80)
+    bad[:, :, ::3] = 0x7FFF
+    q = synth.q_host(37, 1, L, Hq, Hkv, 1)
+    kn, vn = synth.step_kv_host(37, [n], [lab[-1]], L, Hkv)
+    got = []
+    for used in (False, True):
+        c = md.Cache(L, Hq, Hkv, ps, 2, 64, 64, region_aligned_pages=aligned)
+        if persistent:
+            c.debug_set(md.MD_DEBUG_GRID_LIMIT, 128)
+        if used:
+            for part in (slice(0, 150), slice(150, n)):
+                c.append_tokens(1, np.full(part.stop - part.start, 6, np.uint8), k[:, :, part].contiguous(),
+                                bad[:, :, part].contiguous())
+            st, n_ev = c.evict([0, 0])
+            assert st == md.MD_WARN_OVER_BUDGET and n_ev[1] == (n + ps - 1) // ps - 1
+        c.append_tokens(0, lab, k, v)
+        slots = c.get_state(md.MD_STATE_BLOCK_TABLE)[0, :c.query(md.MD_QUERY_PAGES, 0)].long()
+        if entry == "device":
+            out = torch.empty((1, L, Hq, 128), dtype=torch.int16, device="cuda")
+            c.decode_step(1, to_dev(q), to_dev(kn), to_dev(vn), [lab[-1]], out)
+        else:
+            pin = [torch.from_numpy(np.ascontiguousarray(a).view(np.int16)).pin_memory() for a in (q, kn, vn)]
+            out = torch.empty((1, L, Hq, 128), dtype=torch.int16).pin_memory()
+            c.decode_step_host(1, *pin, [lab[-1]], out)
+        assert c.sync() == md.MD_OK
+        got.append((out.cpu(), c.get_state(md.MD_STATE_MASS).view(-1, ps)[slots]))
+        c.close()
+    assert torch.isfinite(got[1][0].view(torch.bfloat16).float()).all()
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
 def test_argument_forms_give_the_same_step():
     """Labels and budgets as exact arrays (taken in place), lists, other
     integer types and strided arrays; host buffers as tensors and as numpy

@@ -79,6 +79,45 @@ def test_noalloc_matches_workspace_path_twice(L, Hq, ps, lengths):
     c.close()
 
 
+@pytest.mark.parametrize("L,Hq,Hkv,ps,lengths", [
+    (1, 16, 2, 16, [1]),
+    (1, 12, 2, 32, [1703, 33]),
+    (2, 16, 2, 16, [430 - 3 * i for i in range(32)]),
+    (1, 16, 2, 16, [20007 - 16 * i for i in range(8)]),      # the persistent kernel
+    (1, 8, 2, 32, [20017 - 32 * i for i in range(8)]),       # the same
+])
+@pytest.mark.parametrize("stale", [0x7FFF, 0x7F80])          # a NaN and an infinity
+def test_noalloc_ignores_what_lies_past_the_cached_tokens(L, Hq, Hkv, ps, lengths, stale):
+    """Slots past a sequence's cached tokens may hold anything: NaN or infinite
+    bits there give the same output and masses, bit for bit, as zeros."""
+    B, P = len(lengths), max(lengths) // ps + 1
+    pages = [(n + ps - 1) // ps for n in lengths]
+    first = np.concatenate([[0], np.cumsum(pages)])
+    g = torch.Generator(device="cuda").manual_seed(47)
+    pool = torch.randn((L, int(first[-1]), Hkv, 2, ps, 128), generator=g, device="cuda").bfloat16().view(torch.int16)
+    bt = torch.zeros((B, P), dtype=torch.int32)
+    for b in range(B):
+        bt[b, :pages[b]] = torch.arange(int(first[b]), int(first[b + 1]))
+    bt = bt.cuda()
+    q = torch.randn((B, L, Hq, 128), generator=g, device="cuda").bfloat16()
+    n_tok = np.array(lengths, np.int32)
+    got = []
+    for bits in (0, stale):
+        for b in range(B):
+            if lengths[b] % ps:
+                pool[:, int(first[b + 1]) - 1, :, :, lengths[b] % ps:] = bits
+        out = torch.zeros((B, L, Hq, 128), dtype=torch.int16, device="cuda")
+        mass = torch.zeros((L * Hkv, int(first[-1]) * ps), device="cuda")
+        st = md.lib().md_attend_mass_noalloc(pool.data_ptr(), bt.data_ptr(), n_tok.ctypes.data, q.data_ptr(),
+                                             out.data_ptr(), mass.data_ptr(), B, L, Hq, Hkv, ps, P, int(first[-1]),
+                                             torch.cuda.current_stream().cuda_stream)
+        assert st == md.MD_OK
+        torch.cuda.synchronize()
+        got.append((out, mass))
+    assert torch.isfinite(got[1][0].view(torch.bfloat16).float()).all()
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
 def test_noalloc_rejects_work_beyond_its_fixed_scratch():
     """Too many (sequence, layer, KV head) items for the fixed array: a clear
     capacity error before anything is launched."""
