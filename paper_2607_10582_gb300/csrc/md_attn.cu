@@ -685,9 +685,9 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
       /* No copy may still be writing this CTA's shared memory when it exits:
        * wait for the last copy issued into every stage. */
       for (int k = (i > S::R ? i - S::R : 0); k < i; ++k)
-        wait_phase(smem_u32(&full[k % S::R]), (k / S::R) & 1, p, 2, false);
+        drain_phase(smem_u32(&full[k % S::R]), (k / S::R) & 1, p, 2);
       for (int k = (nu > 2 ? nu - 2 : 0); k < nu; ++k)
-        wait_phase(smem_u32(&qfull[k & 1]), (k >> 1) & 1, p, 6, false);
+        drain_phase(smem_u32(&qfull[k & 1]), (k >> 1) & 1, p, 6);
     }
     return;
   }

@@ -38,6 +38,20 @@ static __device__ __noinline__ bool wait_phase(uint32_t bar, uint32_t parity, co
   }
 }
 
+/* Waits for a copy that this CTA has issued to land, before the CTA exits: a
+ * copy still in flight would write shared memory that the next CTA owns.  The
+ * limit is not the handle's wait limit, which may be set below the time a copy
+ * takes (1 us at least). */
+constexpr long long DRAIN_LIMIT_NS = 2000000000LL;
+static __device__ __noinline__ void drain_phase(uint32_t bar, uint32_t parity, const AttnBase &p, int diag) {
+  const long long t0 = globaltimer();
+  while (!mbar_try_wait(bar, parity))
+    if (globaltimer() - t0 > DRAIN_LIMIT_NS) {
+      raise_status(p, MD_ERR_DEVICE_TIMEOUT, diag);
+      return;
+    }
+}
+
 /* Address of the 16-byte chunk holding (row, d..d+7) of a stage stored as two
  * 64-column halves of 128-byte rows with the TMA 128-byte swizzle. */
 template <int PS>

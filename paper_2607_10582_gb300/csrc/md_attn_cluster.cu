@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
     }
   }
   if (n < nt)   // a wait ran out: the copies still in flight must land before the CTA exits
-    for (; n < issued; ++n) wait_phase(bar_u32 + (n % STAGES) * 8, (n / STAGES) & 1, p, 2, false);
+    for (; n < issued; ++n) drain_phase(bar_u32 + (n % STAGES) * 8, (n / STAGES) & 1, p, 2);
 
   /* ---- merge the warps: (m, Z, O) of the chunk ---- */
 #pragma unroll

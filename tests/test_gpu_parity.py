@@ -873,3 +873,26 @@ def test_device_wait_timeout_is_reported_not_hung():
     ls2.prefill()
     ls2.decode()
     ls2.observe()
+
+
+@pytest.mark.parametrize("persistent", [0, 1])
+@pytest.mark.parametrize("n", [600, 6000])
+def test_wait_limit_shorter_than_a_copy(persistent, n):
+    """With the smallest wait limit (1 us, less than a copy from HBM may take)
+    a step either finishes or reports the timeout, its copies have landed before
+    the kernel ends, and a new handle over the same memory computes as ever."""
+    w = synth.custom_workload("short", L=2, Hq=16, Hkv=2, page_size=16, lengths=[n, 300], budget_frac=0.5, steps=2,
+                              seed=51)
+    for _ in range(4):
+        ls = Lockstep(w)
+        ls.prefill()
+        ls.gpu.debug_set(md.MD_DEBUG_SPIN_LIMIT_NS, 1000)
+        if persistent:
+            ls.gpu.debug_set(md.MD_DEBUG_GRID_LIMIT, 128)
+        q = synth.q_host(w.seed, 2, 2, 16, 2, 1)
+        kn, vn = synth.step_kv_host(w.seed, ls.pos, [6, 6], 2, 2)
+        out = torch.empty((2, 2, 16, 128), dtype=torch.int16, device="cuda")
+        ls.gpu.decode_step(2, to_dev(q), to_dev(kn), to_dev(vn), [6, 6], out)
+        assert ls.gpu.sync() in (md.MD_OK, md.MD_ERR_DEVICE_TIMEOUT)
+        ls.gpu.close()
+    Lockstep(w).run().check_layout()
