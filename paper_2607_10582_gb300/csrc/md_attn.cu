@@ -141,7 +141,7 @@ __device__ __forceinline__ int load_batch(const AttnParams &p, const Unit &x, in
     const uint8_t *fr = p.page_fill + (size_t)x.b * p.P_max;
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-      fl[k] = k >= cnt ? 0 : (NEW && from + k == last ? p.nt.tail_fill[x.b] : fr[from + k]);
+      fl[k] = k < cnt ? fr[from + k] : 0;
   } else {
 #pragma unroll
     for (int k = 0; k < 8; ++k) fl[k] = 0;
@@ -184,8 +184,7 @@ __device__ __forceinline__ void load_page_ids(const AttnParams &p, const Unit &p
       ph[r] = fl[r] = 0;
       if (q < npg) {
         ph[r] = *(tail && pop >= 0 ? p.nt.free_stack + pop : bt + pv.p0 + q);
-        if (ALIGNED)
-          fl[r] = NEW && tail ? p.nt.tail_fill[pv.b] : p.page_fill[(size_t)pv.b * p.P_max + pv.p0 + q];
+        if (ALIGNED) fl[r] = p.page_fill[(size_t)pv.b * p.P_max + pv.p0 + q];
       }
     }
 #pragma unroll
@@ -487,15 +486,16 @@ __device__ __forceinline__ void single_end(const AttnParams &p, const Unit &un, 
  * every page but the last is full and the fills follow from n_tokens.  ROWS:
  * the masses go to one fp32 row per (layer, KV head) (the no-allocation entry
  * point) instead of the step's fixed-point accumulator.  NEW: the launch
- * also appends the step's new tokens (NewTokens).  Compile-time choices: the
- * end-of-unit code runs once per unit and is often fetched cold, and a runtime
- * test in the page loads made the no-allocation call 3% longer (24 x 999
- * tokens, 16 layers: 60.6 -> 62.5 us). */
+ * also appends the step's new tokens (NewTokens; contiguous pages only).
+ * Compile-time choices: the end-of-unit code runs once per unit and is often
+ * fetched cold, and a runtime test in the page loads made the no-allocation
+ * call 3% longer (24 x 999 tokens, 16 layers: 60.6 -> 62.5 us). */
 template <int PS, int NCW, bool ALIGNED, bool ROWS, bool NEW>
 __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW>::CTAS_PER_SM)
     attn_mass_kernel(const __grid_constant__ AttnParams p,
                      const __grid_constant__ CUtensorMap tmap) {
   using S = AttnShape<PS, NCW>;
+  static_assert(!(ALIGNED && NEW), "with region-aligned pages the append is a launch of its own");
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *ring = smem;
@@ -928,14 +928,13 @@ static cudaError_t prepare_impl() {
 }
 
 /* The instances of one page size: the step's (contiguous or region-aligned
- * pages, with or without the append) and the no-allocation entry point's
- * (contiguous pages, mass rows). */
+ * pages, the former with or without the append) and the no-allocation entry
+ * point's (contiguous pages, mass rows). */
 template <int PS>
 static cudaError_t prepare_all() {
   cudaError_t e = prepare_impl<PS, false, false, false>();
   if (e == cudaSuccess) e = prepare_impl<PS, true, false, false>();
   if (e == cudaSuccess) e = prepare_impl<PS, false, false, true>();
-  if (e == cudaSuccess) e = prepare_impl<PS, true, false, true>();
   if (e == cudaSuccess) e = prepare_impl<PS, false, true, false>();
   return e;
 }
@@ -990,9 +989,7 @@ static cudaError_t launch_ps(const AttnParams &p, const CUtensorMap &tmap, int g
     if (p.page_fill || add) return cudaErrorInvalidValue;
     return launch_impl<PS, false, true, false>(p, tmap, grid, s);
   }
-  if (p.page_fill)
-    return add ? launch_impl<PS, true, false, true>(p, tmap, grid, s)
-               : launch_impl<PS, true, false, false>(p, tmap, grid, s);
+  if (p.page_fill) return add ? cudaErrorInvalidValue : launch_impl<PS, true, false, false>(p, tmap, grid, s);
   return add ? launch_impl<PS, false, false, true>(p, tmap, grid, s)
              : launch_impl<PS, false, false, false>(p, tmap, grid, s);
 }

@@ -795,15 +795,19 @@ md_status begin_step(md_ctx *c, int batch, const uint8_t *new_region_host) {
   return MD_OK;
 }
 
-/* The step's append as a launch of its own, for new K/V that lie in host
- * memory: every layer's rows in one pass over the host link, where the
- * attention units' reads of two short rows each would pay its latency.  With
- * q_src (pinned host memory) the pass brings the query rows as well. */
-md_status append_step(md_ctx *c, int batch, const void *k_new, const void *v_new, const void *q_src, void *q_dst,
-                      size_t q_bytes) {
+/* The step's append in layers [l0, l0 + L) as a launch of its own.  For new K/V
+ * that lie in host memory: all layers' rows in one pass over the host link,
+ * where the attention units' reads of two short rows each would pay its
+ * latency; with q_src (pinned host memory) the pass brings the query rows as
+ * well.  And ahead of the persistent attention kernel, unless that appends
+ * (append_inside). */
+md_status append_step(md_ctx *c, int batch, int l0, int L, const void *k_new, const void *v_new, const void *q_src,
+                      void *q_dst, size_t q_bytes) {
   const md_config &cf = c->cfg;
   AppendStepParams ap;
   ap.to = append_to(c);
+  ap.l0 = l0;
+  ap.L = L;
   ap.k_src = (const uint16_t *)k_new;
   ap.v_src = (const uint16_t *)v_new;
   ap.q_src = (const uint4 *)q_src;
@@ -813,7 +817,7 @@ md_status append_step(md_ctx *c, int batch, const void *k_new, const void *v_new
   ap.insert_step = (int)c->m.t;
   for (int b = 0; b < batch; ++b) {
     ap.tok0[b] = (c->n_pages[b] - 1) * cf.page_size + c->tail_fill[b] - 1;
-    ap.pop[b] = c->tail_pop[b];
+    ap.pop[b] = l0 == 0 ? c->tail_pop[b] : -1;
     ap.regions[b] = (uint8_t)c->tail_region[b];
   }
   cudaEvent_t e0;
@@ -823,8 +827,24 @@ md_status append_step(md_ctx *c, int batch, const void *k_new, const void *v_new
   return e == cudaSuccess ? MD_OK : cuda_fail(c, e, "append launch");
 }
 
+/* Whether the persistent kernel also appends a step's new tokens.  The unit
+ * with a sequence's last page then fetches, patches and writes two rows, about
+ * 0.3 us of a CTA's time per (sequence, layer, KV head) item, against the 2.5
+ * us of a launch of its own: it pays up to 3 items per CTA (2 sequences of
+ * 30,000 tokens in 36 layers, 144 items: 341.5 us, 344 with the launch; 16 of
+ * 500 to 8,000 in 28, 896 items: 316 both; 12 of 1,100, 4 KV heads, 36 layers,
+ * 1,728 items: 157.6 and 154.0; 256 of 300, 18,432 items: 508.5 and 479.4).
+ * Region-aligned pages always take the launch: the producer reads a fill per
+ * page, and telling the last page from the others there slows every page
+ * (22 sequences of 4,160 tokens, 8 layers, 2 steps: 602 and 512 us). */
+bool append_inside(const md_ctx *c, int batch, int layers) {
+  return !c->cfg.region_aligned_pages &&
+         (long long)batch * layers * c->cfg.num_kv_heads <= 3LL * c->grid_limit;
+}
+
 /* Stage 1 over layers [l0, l0 + L); q/out hold q_layers layers.  With k_new
- * the launch also appends the step's new tokens (device rows [batch][L][Hkv][D]). */
+ * the step's new tokens are appended too (device rows [batch][L][Hkv][D]), by
+ * the attention launch or by one ahead of it. */
 md_status run_attention(md_ctx *c, int batch, int l0, int L, int q_layers, const void *q_dev,
                         const void *k_new, const void *v_new, void *out_dev) {
   const md_config &cf = c->cfg;
@@ -890,6 +910,11 @@ md_status run_attention(md_ctx *c, int batch, int l0, int L, int q_layers, const
     e = launch_cluster(base, plan, k_new && l0 > 0, ptr<float>(c, c->lay.scratch), c->tmap_tile, c->stream);
     prof_end(c, STAGE_ATTN, e0);
     return e == cudaSuccess ? MD_OK : cuda_fail(c, e, "attention launch");
+  }
+  if (k_new && !append_inside(c, batch, L)) {
+    const md_status st = append_step(c, batch, l0, L, k_new, v_new, nullptr, nullptr, 0);
+    if (st != MD_OK) return st;
+    memset(&base.nt, 0, sizeof(base.nt));
   }
   AttnParams atp;
   memset(&atp, 0, sizeof(atp));
@@ -993,7 +1018,7 @@ MD_API md_status md_decode_step_host(md_ctx *c, int batch, const void *q_host, c
   if (e != cudaSuccess) return cuda_fail(c, e, "input copy");
   st = begin_step(c, batch, new_region_host);
   if (st != MD_OK) return st;
-  st = append_step(c, batch, vk ? vk : dk, vv ? vv : dv, vq, dq, q_bytes);
+  st = append_step(c, batch, 0, cf.num_layers, vk ? vk : dk, vv ? vv : dv, vq, dq, q_bytes);
   if (st != MD_OK) return st;
   st = run_attention(c, batch, 0, cf.num_layers, cf.num_layers, dq, nullptr, nullptr, vo ? vo : dout);
   if (st != MD_OK) return st;

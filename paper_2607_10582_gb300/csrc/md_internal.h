@@ -71,9 +71,12 @@ struct AppendTo {
   int L, Hkv, ps, P_phys, P_max;
 };
 /* One new token for each of n_seqs sequences (a decode step's append as a
- * launch of its own); k_src, v_src are [n_seqs][L][Hkv][D]. */
+ * launch of its own), in layers [l0, l0 + L); k_src, v_src are
+ * [n_seqs][L][Hkv][D].  Layer 0 opens the pages and starts the tokens' state;
+ * later layers find both. */
 struct AppendStepParams {
   AppendTo to;
+  int l0, L;
   const uint16_t *k_src, *v_src;
   const uint4 *q_src;                    // query rows to bring into the workspace on the way
   uint4 *q_dst;

@@ -80,7 +80,7 @@ __global__ void append_step_kernel(const __grid_constant__ AppendStepParams p) {
   pdl_wait();
   pdl_trigger();
   const AppendTo &d = p.to;
-  const unsigned lh = d.L * d.Hkv, total = p.n_seqs * lh * 32u;
+  const unsigned lh = p.L * d.Hkv, total = p.n_seqs * lh * 32u;
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total + p.q_n; i += gridDim.x * blockDim.x) {
     if (i >= total) {
       p.q_dst[i - total] = p.q_src[i - total];
@@ -89,13 +89,13 @@ __global__ void append_step_kernel(const __grid_constant__ AppendStepParams p) {
     const unsigned w = i;
     const int c = w & 15, kv = (w >> 4) & 1;
     const unsigned x = w >> 5, j = x / lh, r = x - j * lh;
-    const int l = r / d.Hkv, h = r - l * d.Hkv;
+    const int l = p.l0 + r / d.Hkv, h = r % d.Hkv;
     const int tok = p.tok0[j], pg = tok / d.ps, off = tok - pg * d.ps, pop = p.pop[j];
     const int phys = pop < 0 ? d.block_table[(size_t)j * d.P_max + pg] : d.free_stack[pop];
     const uint16_t *src = (kv == 0 ? p.k_src : p.v_src) + (size_t)x * D;
     uint16_t *dst = d.pool + ((((size_t)l * d.P_phys + phys) * d.Hkv + h) * 2 + kv) * (size_t)d.ps * D + (size_t)off * D;
     ((uint4 *)dst)[c] = ((const uint4 *)src)[c];
-    if (r == 0 && kv == 0 && c == 0) {
+    if (p.l0 == 0 && r == 0 && kv == 0 && c == 0) {
       start_token(d, (size_t)phys * d.ps + off, p.regions[j], p.insert_step);
       if (pop >= 0) d.block_table[(size_t)j * d.P_max + pg] = phys;
       d.page_fill[(size_t)j * d.P_max + pg] = (uint8_t)(off + 1);
@@ -105,7 +105,7 @@ __global__ void append_step_kernel(const __grid_constant__ AppendStepParams p) {
 }
 
 cudaError_t launch_append_step(const AppendStepParams &p, cudaStream_t s) {
-  const long long total = (long long)p.n_seqs * p.to.L * p.to.Hkv * 32 + p.q_n;
+  const long long total = (long long)p.n_seqs * p.L * p.to.Hkv * 32 + p.q_n;
   long long blocks = (total + 255) / 256;
   if (blocks > 152 * 16) blocks = 152 * 16;
   return launch_pdl(append_step_kernel, (int)blocks, 256, 0, s, p);
