@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
            * the unit holds its page) into a double-buffered slot */
           const int qs = nu & 1;
           if (nu >= 2) {
-            if (!wait_phase(smem_u32(&qempty[qs]), ((nu >> 1) - 1) & 1, p, 5, true)) {
+            if (!wait_phase(smem_u32(&qempty[qs]), ((nu >> 1) - 1) & 1, p, 5, true, p.spin_limit_ns)) {
               ok = false;
               break;
             }
@@ -655,7 +655,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
           if (k >= cnt) break;
           const int s = i % S::R;
           if (i >= S::R) {
-            if (!wait_phase(smem_u32(&empty[s]), ((i / S::R) - 1) & 1, p, 1, true)) {
+            if (!wait_phase(smem_u32(&empty[s]), ((i / S::R) - 1) & 1, p, 1, true, p.spin_limit_ns)) {
               ok = false;
               break;
             }
@@ -685,9 +685,9 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
       /* No copy may still be writing this CTA's shared memory when it exits:
        * wait for the last copy issued into every stage. */
       for (int k = (i > S::R ? i - S::R : 0); k < i; ++k)
-        drain_phase(smem_u32(&full[k % S::R]), (k / S::R) & 1, p, 2);
+        wait_phase(smem_u32(&full[k % S::R]), (k / S::R) & 1, p, 2, false, DRAIN_LIMIT_NS);
       for (int k = (nu > 2 ? nu - 2 : 0); k < nu; ++k)
-        drain_phase(smem_u32(&qfull[k & 1]), (k >> 1) & 1, p, 6);
+        wait_phase(smem_u32(&qfull[k & 1]), (k >> 1) & 1, p, 6, false, DRAIN_LIMIT_NS);
     }
     return;
   }
@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
     for (int u = blockIdx.x; u < p.total_units; u += gridDim.x, ++k) {
       if (u + (int)gridDim.x >= p.total_units) break;   // the consumers finish the last unit
       const Unit pv = decode_unit(p, u);
-      const bool ok = wait_phase(smem_u32(&cdone[k & 1]), (k >> 1) & 1, p, 8, true);
+      const bool ok = wait_phase(smem_u32(&cdone[k & 1]), (k >> 1) & 1, p, 8, true, p.spin_limit_ns);
       if (!__all_sync(0xffffffffu, ok)) break;
       if (pv.C == 1) {
         single_end<PS, ALIGNED, NCW, 32, ROWS, NEW>(p, pv, k & 1, lane, wm, wl, wf, wO, fs, smem_u32(&mdone[0]));
@@ -749,7 +749,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
     uint32_t qf[8][2];
     {
       const int qs = nunit & 1;
-      if (!wait_phase(smem_u32(&qfull[qs]), (nunit >> 1) & 1, p, 7, true)) aborted = true;
+      if (!wait_phase(smem_u32(&qfull[qs]), (nunit >> 1) & 1, p, 7, true, p.spin_limit_ns)) aborted = true;
       const int mi = lane >> 3, rr = lane & 7;
       const uint32_t qb = sQ_u32 + qs * S::Q_BYTES + rr * (D * 2) + mi * 16;
 #pragma unroll
@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
     /* the score slot is free once the finisher is done with the unit that
      * used it two units ago */
     if (nunit >= 2 && !aborted &&
-        !wait_phase(smem_u32(&fdone[slot]), ((nunit >> 1) - 1) & 1, p, 9, true))
+        !wait_phase(smem_u32(&fdone[slot]), ((nunit >> 1) - 1) & 1, p, 9, true, p.spin_limit_ns))
       aborted = true;
     aborted = __any_sync(0xffffffffu, aborted);   // one decision per warp
     float m0 = NEG_INF, m1 = NEG_INF, l0 = 0.f, l1 = 0.f;
@@ -781,7 +781,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
     for (int jp = j0; jp < npg && !aborted; jp += NCW) {
       const int gi = i_base + jp;
       const int s = gi % S::R;
-      if (!wait_phase(smem_u32(&full[s]), (gi / S::R) & 1, p, 4, true)) {
+      if (!wait_phase(smem_u32(&full[s]), (gi / S::R) & 1, p, 4, true, p.spin_limit_ns)) {
         aborted = true;
         break;
       }
@@ -872,8 +872,9 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
      * has read them; on the CTA's last unit the finisher must be done with
      * everything (its finish area is used below) */
     if (!aborted && nunit >= 1) {
-      const bool okw = last ? wait_phase(smem_u32(&fdone[(nunit - 1) & 1]), ((nunit - 1) >> 1) & 1, p, 9, true)
-                            : wait_phase(smem_u32(&mdone[0]), (nunit - 1) & 1, p, 10, true);
+      const int prev = nunit - 1;
+      const bool okw = last ? wait_phase(smem_u32(&fdone[prev & 1]), (prev >> 1) & 1, p, 9, true, p.spin_limit_ns)
+                            : wait_phase(smem_u32(&mdone[0]), prev & 1, p, 10, true, p.spin_limit_ns);
       if (!okw) aborted = true;
       aborted = __any_sync(0xffffffffu, aborted);
     }

@@ -23,33 +23,24 @@ __device__ __forceinline__ void raise_status(const AttnBase &p, int code, int di
   atomicExch(&p.status[ST_ABORT], 1);
 }
 
+/* The wait for copies that a CTA has issued, before it exits: one still in
+ * flight would write shared memory that the next CTA owns.  Not the handle's
+ * wait limit, which may be set below the time a copy takes (1 us at least). */
+constexpr long long DRAIN_LIMIT_NS = 2000000000LL;
+
 /* Bounded wait on an mbarrier phase; false on abort or timeout. */
 static __device__ __noinline__ bool wait_phase(uint32_t bar, uint32_t parity, const AttnBase &p,
-                                        int diag, bool honour_abort) {
+                                        int diag, bool honour_abort, long long limit_ns) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = globaltimer();
   while (true) {
     if (mbar_try_wait(bar, parity)) return true;
     if (honour_abort && ld_volatile(&p.status[ST_ABORT])) return false;
-    if (globaltimer() - t0 > p.spin_limit_ns) {
+    if (globaltimer() - t0 > limit_ns) {
       raise_status(p, MD_ERR_DEVICE_TIMEOUT, diag);
       return false;
     }
   }
-}
-
-/* Waits for a copy that this CTA has issued to land, before the CTA exits: a
- * copy still in flight would write shared memory that the next CTA owns.  The
- * limit is not the handle's wait limit, which may be set below the time a copy
- * takes (1 us at least). */
-constexpr long long DRAIN_LIMIT_NS = 2000000000LL;
-static __device__ __noinline__ void drain_phase(uint32_t bar, uint32_t parity, const AttnBase &p, int diag) {
-  const long long t0 = globaltimer();
-  while (!mbar_try_wait(bar, parity))
-    if (globaltimer() - t0 > DRAIN_LIMIT_NS) {
-      raise_status(p, MD_ERR_DEVICE_TIMEOUT, diag);
-      return;
-    }
 }
 
 /* Address of the 16-byte chunk holding (row, d..d+7) of a stage stored as two

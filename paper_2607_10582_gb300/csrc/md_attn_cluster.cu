@@ -175,7 +175,11 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
   int n = 0;
   for (; n < nt; ++n) {
     const uint32_t st = ring_u32 + (n % STAGES) * TILE_BYTES;
-    if (!__all_sync(0xffffffffu, wait_phase(bar_u32 + (n % STAGES) * 8, (n / STAGES) & 1, p, 4, false))) break;
+    /* the call, and the fetch of its code, only if the copy has not landed in
+     * the first try: 32 sequences of 430 tokens layer by layer 229.9 -> 225.7 us */
+    const uint32_t bar = bar_u32 + (n % STAGES) * 8, parity = (n / STAGES) & 1;
+    const bool landed = mbar_try_wait(bar, parity) || wait_phase(bar, parity, p, 4, false, p.spin_limit_ns);
+    if (!__all_sync(0xffffffffu, landed)) break;
     if (LONG && n > 0 && n % 32 == 0) {
       id = id2;
       fill = fill2;
@@ -257,7 +261,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 2)
     }
   }
   if (n < nt)   // a wait ran out: the copies still in flight must land before the CTA exits
-    for (; n < issued; ++n) drain_phase(bar_u32 + (n % STAGES) * 8, (n / STAGES) & 1, p, 2);
+    for (; n < issued; ++n) wait_phase(bar_u32 + (n % STAGES) * 8, (n / STAGES) & 1, p, 2, false, DRAIN_LIMIT_NS);
 
   /* ---- merge the warps: (m, Z, O) of the chunk ---- */
 #pragma unroll
