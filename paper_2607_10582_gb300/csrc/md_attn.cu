@@ -547,15 +547,12 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
   }
   __syncthreads();
   /* The kernel ahead in the stream may still be writing the block table, the
-   * pool or (a step with host buffers) the query rows: every thread waits for
-   * it before its first global access.  Only the no-allocation call, whose
-   * cache nothing of this library writes, lets the producer's issuing lane
-   * start its first unit's copies before. */
-  const bool issuer = warp == 0 && lane == 0;
-  if (!issuer) {
-    pdl_wait();
-    pdl_trigger();
-  }
+   * pool or the query rows: every thread waits for it before its first global
+   * access.  (Copies before the wait, of a first unit's query rows and pages
+   * below the sequence's last one, changed no launch that takes this kernel by
+   * more than 0.5%.) */
+  pdl_wait();
+  pdl_trigger();
 
   if (warp == 0) {
     /* ------------------------------------------------------- producer ---- */
@@ -580,38 +577,8 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
       if (u < p.total_units) {
         un = decode_unit(p, u);
         pb = un.p0;
+        cnt = pb < un.p1 ? load_batch<ALIGNED, NEW>(p, un, pb, un.p1, ph, fl) : 0;
       }
-      if (u < p.total_units && ROWS) {
-        /* before the wait: the first unit's query rows (the caller's) and,
-         * when the unit is its item's only chunk, its pages below the
-         * sequence's last one, at most one per stage (measured on a GB300:
-         * 3 us off a 24 us step with single-chunk items; with split items the
-         * early pages made the launch 2 us longer, so they wait there) */
-        mbar_arrive_expect_tx(smem_u32(&qfull[0]), G * D * 2);
-        bulk_load(sQ_u32, p.q + (((size_t)un.b * p.q_layers + (un.l - p.l0)) * p.Hq + (size_t)un.kvh * G) * D,
-                  G * D * 2, smem_u32(&qfull[0]));
-        nu = 1;
-        const int early_end = un.C == 1 ? min(min(un.p1, un.p0 + S::R), p.n_pages[un.b] - 1) : un.p0;
-        for (pb = un.p0; pb < early_end; pb += 8) {
-          cnt = load_batch<ALIGNED, NEW>(p, un, pb, early_end, ph, fl);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            if (k >= cnt) break;
-            const int s = i;   // i < R: every stage is still empty
-            const int row = (((un.l * p.P_phys + ph[k]) * p.Hkv + un.kvh) * 2) * PS;
-            const uint32_t st = ring_u32 + s * S::STAGE_BYTES;
-            if (ALIGNED) fillbuf[s] = fl[k];
-            mbar_arrive_expect_tx(smem_u32(&full[s]), S::STAGE_BYTES);
-            tma_load_2d(st, &tmap, 0, row, smem_u32(&full[s]), pol);
-            tma_load_2d(st + S::HALF_BYTES, &tmap, 64, row, smem_u32(&full[s]), pol);
-            ++i;
-          }
-        }
-        pb = un.p0 + i;
-      }
-      pdl_wait();
-      pdl_trigger();
-      if (u < p.total_units) cnt = pb < un.p1 ? load_batch<ALIGNED, NEW>(p, un, pb, un.p1, ph, fl) : 0;
       while (u < p.total_units && ok) {
         Unit nx = un;
         int npb = pb + 8, nxu = u, cntn = 0;
@@ -624,7 +591,7 @@ __global__ void __launch_bounds__(AttnShape<PS, NCW>::THREADS, AttnShape<PS, NCW
           }
         }
         if (nxu < p.total_units) cntn = load_batch<ALIGNED, NEW>(p, nx, npb, nx.p1, phn, fln);
-        if (pb == un.p0 && (!ROWS || u != (int)blockIdx.x)) {   // ROWS: the first unit's went out before the wait
+        if (pb == un.p0) {
           /* the unit's G query rows (and the new token's K and V rows, where
            * the unit holds its page) into a double-buffered slot */
           const int qs = nu & 1;
