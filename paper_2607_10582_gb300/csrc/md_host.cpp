@@ -1265,14 +1265,17 @@ MD_API md_status md_get_state(md_ctx *c, int what, void *dst, size_t bytes) {
   size_t off, n;
   if (!state_array(c, what, &off, &n)) return fail(c, MD_ERR_INVALID_ARG, "unknown state array");
   if (bytes != n) return fail(c, MD_ERR_INVALID_ARG, "state array is %zu bytes, not %zu", n, bytes);
-  /* by a kernel where dst is this device's memory and aligned for it; the
-   * K/V pool and other large arrays are left to the copy engine */
+  /* by a kernel where dst is this device's memory and aligned for it, and this
+   * device is the current one (a kernel cannot be launched on another device's
+   * stream, a copy can); the K/V pool and other large arrays are left to the
+   * copy engine */
   bool here = n <= COPY_KERNEL_BYTES && n % 16 == 0 && ((uintptr_t)dst & 15) == 0;
   if (here) {
     cudaPointerAttributes at;
-    here = cudaPointerGetAttributes(&at, dst) == cudaSuccess;
+    int current = -1;
+    here = cudaGetDevice(&current) == cudaSuccess && cudaPointerGetAttributes(&at, dst) == cudaSuccess;
     if (!here) cudaGetLastError();
-    here = here && at.type == cudaMemoryTypeDevice && at.device == c->device;
+    here = here && current == c->device && at.type == cudaMemoryTypeDevice && at.device == c->device;
   }
   cudaError_t e;
   if (here)
