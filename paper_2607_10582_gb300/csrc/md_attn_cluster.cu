@@ -478,7 +478,7 @@ cudaError_t cluster_prepare() {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (dev < 0 || dev >= 64) return cudaSuccess;   // no table: cluster_plan keeps the persistent kernel
   ClusterSlots &g = g_slots[dev];
   std::lock_guard<std::mutex> lock(g_slots_mu);
   if (g.ready.load(std::memory_order_relaxed)) return cudaSuccess;

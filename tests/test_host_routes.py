@@ -32,3 +32,15 @@ def test_state_reads_from_another_current_device(tmp_path):
                             "-Wl,--unresolved-symbols=ignore-all"], exe)
     assert lines == ["get_state current 0 owner 0: 0 kernel", "get_state current 0 owner 1: 0 copy",
                      "get_state current 1 owner 0: 0 copy", "get_state current 1 owner 1: 0 copy"]
+
+
+def test_device_ordinals_past_the_cluster_table(tmp_path):
+    """Devices from ordinal 64 on have no table of cluster slots: the cluster
+    kernel's preparation succeeds there all the same, and every launch takes the
+    persistent kernel."""
+    nvcc = shutil.which("nvcc") or pytest.skip("no nvcc")
+    exe = str(tmp_path / "device_ordinal")
+    lines = _run(tmp_path, [nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-std=c++17", "-O1",
+                            "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include"), "-o", exe,
+                            os.path.join(ROOT, "tests", "c", "device_ordinal.cu")], exe)
+    assert lines == [f"device {d}: 0, 0" for d in (64, 127, 500)]
