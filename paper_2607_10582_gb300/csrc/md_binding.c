@@ -84,8 +84,10 @@ static int host_ptr(PyObject *o, void **out) {
 }
 
 /* A one-dimensional C-contiguous buffer of items with this format: 1 and the
- * view (to be released), 0 if it is something else, never an exception. */
+ * view (to be released), 0 if it is something else, never an exception.  Not a
+ * byte string: the caller's conversion reads its bytes as text. */
 static int host_view(PyObject *o, char format, Py_ssize_t item, int writable, Py_buffer *view) {
+  if (PyBytes_Check(o)) return 0;
   if (PyObject_GetBuffer(o, view, PyBUF_C_CONTIGUOUS | PyBUF_FORMAT | (writable ? PyBUF_WRITABLE : 0)) != 0) {
     PyErr_Clear();
     return 0;
