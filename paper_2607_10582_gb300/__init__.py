@@ -243,6 +243,13 @@ class Cache:
         except Exception:
             pass
 
+    def _labels(self, regions, batch: int):
+        """The labels as an array the library may read `batch` entries of."""
+        regs, p = _host(regions, np.uint8)
+        if regs.size < batch <= self.max_batch:
+            raise MemDecayError(MD_ERR_INVALID_ARG, f"{regs.size} labels for a batch of {batch}")
+        return regs, p
+
     # -- calls --
     def set_region_params(self, region: int, base: float, half_life: float, pinned: bool):
         return self._check(lib().md_set_region_params(self.h, region, base, half_life, int(pinned)))
@@ -258,7 +265,7 @@ class Cache:
         st = self._b.decode_step(self._hv, batch, q, k_new, v_new, new_regions, out)
         if st is not None:
             return self._check(st)
-        regs, rp = _host(new_regions, np.uint8)
+        regs, rp = self._labels(new_regions, batch)
         return self._check(lib().md_decode_step(self.h, batch, _ptr(q), _ptr(k_new), _ptr(v_new), rp, _ptr(out)))
 
     def decode_step_host(self, batch: int, q, k_new, v_new, new_regions, out):
@@ -268,7 +275,7 @@ class Cache:
         st = self._b.decode_step_host(self._hv, batch, q, k_new, v_new, new_regions, out)
         if st is not None:
             return self._check(st)
-        regs, rp = _host(new_regions, np.uint8)
+        regs, rp = self._labels(new_regions, batch)
         return self._check(lib().md_decode_step_host(self.h, batch, _hptr(q), _hptr(k_new), _hptr(v_new), rp,
                                                      _hptr(out)))
 
@@ -276,7 +283,7 @@ class Cache:
         st = self._b.decode_layer(self._hv, layer, batch, q, k_new, v_new, new_regions, out)
         if st is not None:
             return self._check(st)
-        regs, rp = _host(new_regions, np.uint8)
+        regs, rp = self._labels(new_regions, batch if layer == 0 else 0)
         return self._check(lib().md_decode_layer(self.h, layer, batch, _ptr(q), _ptr(k_new), _ptr(v_new), rp,
                                                  _ptr(out)))
 

@@ -98,6 +98,14 @@ static int host_view(PyObject *o, char format, Py_ssize_t item, int writable, Py
   return 0;
 }
 
+/* The labels of a step: one per sequence of the batch at least. */
+static int label_view(PyObject *o, int batch, Py_buffer *view) {
+  if (!host_view(o, 'B', 1, 0, view)) return 0;
+  if (view->shape[0] >= batch) return 1;
+  PyBuffer_Release(view);
+  return 0;
+}
+
 static int as_int(PyObject *o, int *out) {
   const long long v = PyLong_AsLongLong(o);
   if (v == -1 && PyErr_Occurred()) return -1;
@@ -120,7 +128,7 @@ static PyObject *decode_step(PyObject *self, PyObject *const *a, Py_ssize_t n) {
   if (arity(n, 7) || dev_ptr(a[0], &h) || as_int(a[1], &batch) || dev_ptr(a[2], &q) || dev_ptr(a[3], &k) ||
       dev_ptr(a[4], &v) || dev_ptr(a[6], &out))
     return NULL;
-  if (!host_view(a[5], 'B', 1, 0, &regs)) Py_RETURN_NONE;
+  if (!label_view(a[5], batch, &regs)) Py_RETURN_NONE;
   Py_BEGIN_ALLOW_THREADS
   st = f_decode_step((md_ctx *)h, batch, q, k, v, (const uint8_t *)regs.buf, out);
   Py_END_ALLOW_THREADS
@@ -140,7 +148,7 @@ static PyObject *decode_step_host(PyObject *self, PyObject *const *a, Py_ssize_t
     if (ok < 0) return NULL;
     if (ok == 0) Py_RETURN_NONE;
   }
-  if (!host_view(a[5], 'B', 1, 0, &regs)) Py_RETURN_NONE;
+  if (!label_view(a[5], batch, &regs)) Py_RETURN_NONE;
   Py_BEGIN_ALLOW_THREADS
   st = f_decode_step_host((md_ctx *)h, batch, x[0], x[1], x[2], (const uint8_t *)regs.buf, x[3]);
   Py_END_ALLOW_THREADS
@@ -156,7 +164,7 @@ static PyObject *decode_layer(PyObject *self, PyObject *const *a, Py_ssize_t n) 
   if (arity(n, 8) || dev_ptr(a[0], &h) || as_int(a[1], &layer) || as_int(a[2], &batch) || dev_ptr(a[3], &q) ||
       dev_ptr(a[4], &k) || dev_ptr(a[5], &v) || dev_ptr(a[7], &out))
     return NULL;
-  if (!host_view(a[6], 'B', 1, 0, &regs)) Py_RETURN_NONE;
+  if (!label_view(a[6], layer == 0 ? batch : 0, &regs)) Py_RETURN_NONE;   // later layers read none
   Py_BEGIN_ALLOW_THREADS
   st = f_decode_layer((md_ctx *)h, layer, batch, q, k, v, (const uint8_t *)regs.buf, out);
   Py_END_ALLOW_THREADS
