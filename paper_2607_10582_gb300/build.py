@@ -1,8 +1,9 @@
 """In-tree build of libmemdecay.so for sm_103a (nvcc; no cmake).
 
 The translation units compile in parallel, then link into one shared library
-next to this file; the Python module of the per-step calls (_calls.so, plain
-C) lands beside it.  Run as a module or call build()."""
+next to this file; the Python module of the per-step calls (_calls, plain C,
+named for the interpreter) lands beside it, unless Python's headers are missing:
+those calls then go through ctypes.  Run as a module or call build()."""
 from __future__ import annotations
 
 import os
@@ -15,7 +16,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB_PATH = os.path.join(HERE, "libmemdecay.so")
-BINDING_PATH = os.path.join(HERE, "_calls.so")
+BINDING_PATH = os.path.join(HERE, "_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
 OBJ_DIR = os.path.join(HERE, "_build")
 SOURCES = ["md_host.cpp", "md_attn.cu", "md_attn_cluster.cu", "md_state.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -30,9 +31,17 @@ def _deps():
     return files
 
 
+def python_include():
+    """The folder of Python.h, or None."""
+    path = sysconfig.get_paths()["include"]
+    return path if os.path.exists(os.path.join(path, "Python.h")) else None
+
+
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) -> str:
     newest = max(os.path.getmtime(p) for p in _deps())
-    if not force and all(os.path.exists(p) and os.path.getmtime(p) >= newest for p in (LIB_PATH, BINDING_PATH)):
+    include = python_include()
+    made = (LIB_PATH, BINDING_PATH) if include else (LIB_PATH,)
+    if not force and all(os.path.exists(p) and os.path.getmtime(p) >= newest for p in made):
         return LIB_PATH
     os.makedirs(OBJ_DIR, exist_ok=True)
 
@@ -51,7 +60,9 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
         return obj
 
     def compile_binding():
-        cmd = ["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", INCLUDE,
+        if not include:
+            return
+        cmd = ["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", include, "-I", INCLUDE,
                os.path.join(CSRC, "md_binding.c"), "-o", BINDING_PATH + ".tmp", "-ldl"]
         if verbose:
             print(" ".join(cmd), flush=True)
