@@ -302,7 +302,8 @@ md_status md_profile_read(md_ctx *ctx, double *ms_per_stage, int64_t *launches_p
                           int n_stages);
 
 /* Test and tuning support.  GRID_LIMIT, FORCE_CHUNKS and EXTRA_ARRIVALS keep
- * the persistent attention kernel, which they are about.
+ * the persistent attention kernel, which they are about.  CLUSTER_FORM takes
+ * the cluster kernel in one form, where none of those three is set.
  *   MD_DEBUG_SPIN_LIMIT_NS    limit of each device-side wait (default 2e9)
  *   MD_DEBUG_EXTRA_ARRIVALS   extra arrivals the attention exchange waits for
  *                             on its next launch (a wait nothing completes;
@@ -322,7 +323,13 @@ md_status md_profile_read(md_ctx *ctx, double *ms_per_stage, int64_t *launches_p
  *   MD_DEBUG_ZERO_COPY        1 (default): md_decode_step_host uses the K/V
  *                             and output buffers in place where the device
  *                             reaches them; 0: it copies every buffer
- *                             through the workspace */
+ *                             through the workspace
+ *   MD_DEBUG_CLUSTER_FORM     0 (default): the kernel and its form are chosen
+ *                             by cost; else C + 256 * W + 65536 * S: clusters
+ *                             of C CTAs (1, 2, 4, 8 or 16) of W warps (4 or 8)
+ *                             per item, scores in shared memory (S = 0) or in
+ *                             scratch (1).  A step that cannot take the form
+ *                             fails with MD_ERR_CUDA. */
 enum {
   MD_DEBUG_SPIN_LIMIT_NS = 0,
   MD_DEBUG_EXTRA_ARRIVALS = 1,
@@ -330,7 +337,8 @@ enum {
   MD_DEBUG_UNIT_OVERHEAD = 3,
   MD_DEBUG_FORCE_CHUNKS = 4,
   MD_DEBUG_COMBINE_OVERHEAD = 5,
-  MD_DEBUG_ZERO_COPY = 6
+  MD_DEBUG_ZERO_COPY = 6,
+  MD_DEBUG_CLUSTER_FORM = 7
 };
 md_status md_debug_set(md_ctx *ctx, int key, int64_t value);
 

@@ -582,6 +582,21 @@ ClusterPlan cluster_plan(const AttnBase &p, size_t scratch_floats) {
   return best;
 }
 
+ClusterPlan cluster_form(const AttnBase &p, size_t scratch_floats, int C, int warps, bool spill) {
+  ClusterPlan f;
+  int T = 1;
+  for (int b = 0; b < p.n_seqs; ++b) T = std::max(T, seq_tiles(p, b));
+  const int n = ((T + C - 1) / C + warps - 1) / warps;
+  const size_t ctas = (size_t)p.n_seqs * p.L_launch * p.Hkv * C;
+  if (spill ? ctas * warps * n * TILE * GP > scratch_floats : n > 32 || cluster_smem(warps, C, n) > CLUSTER_SMEM)
+    return f;
+  f.C = C;
+  f.warps = warps;
+  f.warp_tiles = n;
+  f.spill = spill;
+  return f;
+}
+
 template <int NW, bool LONG>
 static cudaError_t launch_warps(const cudaLaunchConfig_t &cfg, const ClusterParams &p, const CUtensorMap &tmap) {
   if (!p.mass_acc)

@@ -69,6 +69,7 @@ struct md_ctx {
   int unit_overhead_kib = 112;   // planner: per-unit cost, as KiB of K/V streamed
   int combine_overhead_kib = 192;   // planner: cost of a split into several chunks per item
   int force_chunks = 0;      // planner: 0 = choose
+  int cluster_form = 0;      // MD_DEBUG_CLUSTER_FORM: 0 = by cost
   /* the planner's last choice of pages per chunk, reused while its inputs
    * (batch, layers, knobs, pages per sequence) repeat */
   std::vector<int> plan_pages;
@@ -902,7 +903,12 @@ md_status run_attention(md_ctx *c, int batch, int l0, int L, int q_layers, const
   }
   /* the debug knobs of the persistent kernel's planner and exchange keep that kernel */
   const bool knobs = c->grid_cap > 0 || c->force_chunks > 0 || c->extra_arrivals > 0;
-  const ClusterPlan plan = knobs ? ClusterPlan{} : cluster_plan(base, (size_t)MAX_GRID * 2 * c->lay.scratch_tokens * GP);
+  const size_t scratch = (size_t)MAX_GRID * 2 * c->lay.scratch_tokens * GP;
+  const int form = knobs ? 0 : c->cluster_form;
+  const ClusterPlan plan = knobs  ? ClusterPlan{}
+                           : form ? cluster_form(base, scratch, form & 255, (form >> 8) & 255, form >> 16)
+                                  : cluster_plan(base, scratch);
+  if (form && plan.C == 0) return cuda_fail(c, cudaErrorInvalidConfiguration, "cluster form");
   cudaEvent_t e0;
   cudaError_t e;
   if (plan.C > 0) {
@@ -1479,6 +1485,13 @@ MD_API md_status md_debug_set(md_ctx *c, int key, int64_t value) {
   if (key == MD_DEBUG_ZERO_COPY) {
     if (value != 0 && value != 1) return fail(c, MD_ERR_INVALID_ARG, "zero-copy switch must be 0 or 1");
     c->zero_copy = (int)value;
+    return MD_OK;
+  }
+  if (key == MD_DEBUG_CLUSTER_FORM) {
+    const int64_t C = value & 255, warps = (value >> 8) & 255, spill = value >> 16;
+    if (value != 0 && (C < 1 || C > MAX_CLUSTER || (C & (C - 1)) || (warps != 4 && warps != 8) || spill < 0 || spill > 1))
+      return fail(c, MD_ERR_INVALID_ARG, "unknown cluster form");
+    c->cluster_form = (int)value;
     return MD_OK;
   }
   if (key == MD_DEBUG_COMBINE_OVERHEAD) {

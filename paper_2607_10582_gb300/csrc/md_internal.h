@@ -194,6 +194,8 @@ struct ClusterPlan {
 };
 cudaError_t cluster_prepare();
 ClusterPlan cluster_plan(const AttnBase &p, size_t scratch_floats);
+/* One form (C = 0: the launch cannot take it); p as for cluster_plan. */
+ClusterPlan cluster_form(const AttnBase &p, size_t scratch_floats, int C, int warps, bool spill);
 cudaError_t launch_cluster(const AttnBase &p, const ClusterPlan &plan, bool early, float *scratch,
                            const CUtensorMap &tmap, cudaStream_t s);
 /* The tensor maps of the K/V pool (encode: the driver's cuTensorMapEncodeTiled). */

@@ -15,6 +15,7 @@ if not torch.cuda.is_available():  # pragma: no cover - GPU tests only run on th
 import paper_2607_10582_gb300 as md  # noqa: E402
 import synth  # noqa: E402
 from paper_2607_10582_gb300 import build as mdbuild  # noqa: E402
+from tests.attention_shapes import CLUSTER  # noqa: E402
 from tests.gpu_harness import TOL_O_ABS, Lockstep, to_dev  # noqa: E402
 
 mdbuild.build()
@@ -407,26 +408,138 @@ def test_entry_points_mixed_step_by_step():
     ls.check_layout()
 
 
-@pytest.mark.parametrize("L,Hq,Hkv,ps,lengths,aligned", [
-    (1, 8, 1, 16, [15], 0),                                  # one tile, one CTA
-    (1, 3, 1, 16, [431], 0),                                 # clusters of 8, G = 3 padded heads
-    (1, 16, 2, 32, [1, 17, 4095], 0),                        # clusters of 16: most chunks of the short ones are empty
-    (2, 28, 4, 32, [1000] * 3 + [33], 1),                    # region-aligned pages, half-empty second tiles
-    (1, 12, 2, 16, [1500 + 16 * i for i in range(12)], 0),   # clusters of CTAs of 8 warps
-    (2, 16, 2, 16, [300 + 7 * i for i in range(40)], 0),     # one CTA per item, more than one wave
-    (3, 5, 1, 16, [1790 - 25 * i for i in range(60)], 0),    # the same with 8 warps
-    (1, 16, 2, 32, [20000, 17, 9001], 0),                    # spilled scores, page ids in several batches
-    (2, 8, 2, 16, [6100, 4000, 5999], 1),                    # the same with region-aligned pages
-    (8, 7, 1, 16, [3500 + 50 * i for i in range(12)], 0),    # spilled scores with 4 warps
-])
+@pytest.mark.parametrize("L,Hq,Hkv,ps,lengths,aligned", [shape for shape, _ in CLUSTER])
 def test_cluster_attention_follows_the_oracle(L, Hq, Hkv, ps, lengths, aligned):
-    """Launch shapes that take the cluster attention kernel in each of its
-    forms, with sizes at the edges of tiles, warps and chunks."""
+    """Launch shapes that take the cluster attention kernel by themselves, with
+    sizes at the edges of tiles, warps and chunks."""
     w = synth.custom_workload("cluster", L=L, Hq=Hq, Hkv=Hkv, page_size=ps, lengths=lengths, budget_frac=0.7,
                               steps=3, seed=41, structured=True)
     w.extra["region_aligned"] = bool(aligned)
     ls = Lockstep(w).run()
     ls.check_layout()
+
+
+@pytest.mark.parametrize("C,warps,spill,n", [
+    (1, 4, 0, 1500), (2, 4, 0, 1500), (8, 4, 0, 1500), (16, 4, 0, 3000),
+    (1, 8, 0, 2200), (4, 8, 0, 2200), (16, 8, 0, 5000),
+    # scores in scratch: 47 and 35 tiles per warp of 4, 34 of 8 (page ids come 32
+    # at a time; the new token is on the last tile), few tiles, and none
+    (1, 4, 1, 3000), (2, 4, 1, 4400), (1, 8, 1, 4340), (8, 4, 1, 900), (16, 8, 1, 5000),
+])
+@pytest.mark.parametrize("ps,aligned", [(16, 0), (32, 0), (16, 1), (32, 1)])
+def test_every_cluster_form_follows_the_oracle(C, warps, spill, n, ps, aligned):
+    """Every form of the cluster kernel on the same kinds of batch (a step at
+    once and layer by layer): one whose sequences fill most chunks, one that
+    leaves most of them empty."""
+    w = synth.custom_workload("form", L=2, Hq=12, Hkv=2, page_size=ps, lengths=[n, 17, n // 3, 1], budget_frac=0.9,
+                              steps=2, seed=43, structured=True)
+    w.extra["region_aligned"] = bool(aligned)
+    ls = Lockstep(w)
+    ls.gpu.debug_set(md.MD_DEBUG_CLUSTER_FORM, C + 256 * warps + 65536 * spill)
+    ls.prefill()
+    for entry in ("device", "layers"):
+        ls.decode(entry=entry)
+        ls.observe()
+    ls.check_layout()
+
+
+def test_cluster_form_that_does_not_fit_fails():
+    """A forced form whose scores fit neither shared memory nor, spilled, the
+    scratch is an error of the step, not another form."""
+    w = synth.custom_workload("nofit", L=1, Hq=4, Hkv=1, page_size=16, lengths=[3000], budget_frac=1.0, steps=1, seed=44)
+    ls = Lockstep(w)
+    ls.prefill()
+    ls.gpu.debug_set(md.MD_DEBUG_CLUSTER_FORM, 1 + 256 * 4)
+    with pytest.raises(md.MemDecayError) as e:
+        ls.decode()
+    assert e.value.status == md.MD_ERR_CUDA
+
+
+@pytest.mark.parametrize("Hq,Hkv,ps,lengths,aligned,window", [
+    (16, 2, 16, [37, 1300, 5003], 0, 1),
+    (12, 2, 32, [700, 2100], 0, 3),
+    (2, 2, 16, [900, 2600], 0, 1),
+    (16, 2, 16, [700, 1900, 0], 1, 1),
+    (12, 2, 32, [1500, 33], 1, 2),
+])
+@pytest.mark.parametrize("entry", ["device", "host", "layers", "mixed"])
+def test_persistent_attention_follows_the_oracle(Hq, Hkv, ps, lengths, aligned, window, entry):
+    """The persistent kernel (kept by the grid limit, here all that fit) on
+    shapes that take the cluster kernel by themselves: both page sizes,
+    contiguous and region-aligned pages, appending inside the launch and behind
+    an append launch."""
+    w = synth.custom_workload("persistent", L=3, Hq=Hq, Hkv=Hkv, page_size=ps, lengths=lengths, budget_frac=0.5,
+                              steps=12, seed=45, window_k=window, structured=True)
+    w.extra["region_aligned"] = bool(aligned)
+    ls = Lockstep(w)
+    ls.gpu.debug_set(md.MD_DEBUG_GRID_LIMIT, 512)
+    ls.prefill()
+    for s in range(w.steps):
+        ls.decode(entry=("device", "host", "layers")[s % 3] if entry == "mixed" else entry,
+                  regions=[[6, 2][s // 2 % 2]] * w.B)
+        if (s + 1) % window == 0:
+            ls.observe()
+    ls.check_layout()
+
+
+@pytest.mark.parametrize("ps,aligned,window", [(16, 0, 1), (32, 0, 3), (32, 1, 1), (16, 1, 2)])
+@pytest.mark.parametrize("kernel", ["by cost", "8 warps", "scratch", "persistent"])
+def test_calls_back_to_back_give_what_calls_one_by_one_give(ps, aligned, window, kernel):
+    """Layer calls, whole steps and evictions issued with nothing between them,
+    on tensors prepared beforehand: launches overlap (layers after the first copy
+    K/V before the layer ahead has ended).  Outputs, the step's mass and the
+    state are the same bits as with a synchronisation after every call."""
+    L, Hq, Hkv, steps = 4, 16, 2, 12
+    lengths = [430, 1, 0, 811, ps * 9, 250]
+    B = len(lengths)
+    rng = np.random.default_rng(53)
+    labels = [np.sort(rng.integers(0, 7, n)).astype(np.uint8) for n in lengths]
+    kv = [[to_dev(x) for x in synth.kv_host(53, b, L, Hkv, 0, n, labels[b])] for b, n in enumerate(lengths)]
+    new = [np.where(rng.random(B) < 0.3, rng.integers(1, 7, B), 6).astype(np.uint8) for _ in range(steps)]
+    x = [[to_dev(t) for t in (synth.q_host(53, B, L, Hq, Hkv, s + 1), *synth.step_kv_host(
+        53, [n + s for n in lengths], new[s], L, Hkv))] for s in range(steps)]
+    rows = [[[t[:, l].contiguous() for t in x[s]] for l in range(L)] for s in range(steps)]
+    budget = np.array([max(1, (n + ps - 1) // ps - 3) for n in lengths], np.int32)
+    got = []
+    for wait in (False, True):
+        c = md.Cache(L, Hq, Hkv, ps, B, 100, 100 * B, region_aligned_pages=aligned)
+        if kernel == "persistent":
+            c.debug_set(md.MD_DEBUG_GRID_LIMIT, 512)
+        elif kernel != "by cost":
+            c.debug_set(md.MD_DEBUG_CLUSTER_FORM, 1 + 256 * 8 if kernel == "8 warps" else 2 + 256 * 4 + 65536)
+        for r in range(7):
+            c.set_region_params(r, 1.0 - 0.1 * r, 20.0, r == 0)
+        for b in range(B):
+            if lengths[b]:
+                c.append_tokens(b, labels[b], *kv[b])
+        out = torch.zeros((steps, L, B, Hq, 128), dtype=torch.int16, device="cuda")
+        whole = torch.zeros((steps, B, L, Hq, 128), dtype=torch.int16, device="cuda")
+        masses = []
+        torch.cuda.synchronize()
+        for s in range(steps):
+            if s % 4 == 3:
+                c.decode_step(B, *x[s], new[s], whole[s])
+            else:
+                for l in range(L):
+                    c.decode_layer(l, B, *rows[s][l], new[s], out[s, l])
+                    if wait:
+                        torch.cuda.synchronize()
+            if wait:
+                torch.cuda.synchronize()
+            masses.append(c.get_state(md.MD_STATE_MASS))
+            if (s + 1) % window == 0:
+                c.evict(budget)
+                if wait:
+                    torch.cuda.synchronize()
+        assert c.sync() == md.MD_OK
+        used = torch.cat([c.get_state(md.MD_STATE_BLOCK_TABLE)[b, :c.query(md.MD_QUERY_PAGES, b)] for b in range(B)])
+        got.append([out, whole, *masses, *[c.get_state(k) for k in (
+            md.MD_STATE_BLOCK_TABLE, md.MD_STATE_FREE, md.MD_STATE_PAGE_FILL, md.MD_STATE_SEQ_TOKENS)]] +
+            [c.get_state(k).view(-1, ps)[used.long()] for k in (
+                md.MD_STATE_REGION, md.MD_STATE_A, md.MD_STATE_T_REF, md.MD_STATE_AHAT)])
+        c.close()
+    for i, (a, b) in enumerate(zip(*got)):
+        assert torch.equal(a, b), i
 
 
 @pytest.mark.parametrize("n", [40, 900])
@@ -455,10 +568,14 @@ def test_one_launch_observation_selects_what_the_two_kernels_select(ps, aligned,
     """A batch of short sequences, scored and selected in one launch, against
     the same batch with the calibration histogram on, which takes the two
     kernels: token state, page scores, tables, fills, counts and evicted pages
-    bit for bit.  Pages at the ends of warps and of the kernel's range, none,
-    one, several and all evictable pages evicted, equal scores (b = 0 and no
-    attention weight)."""
+    bit for bit.  Pages at the ends of warps and of the kernel's range (256
+    pages, 4,096 slots), none, one, several and all evictable pages evicted,
+    equal scores (b = 0 and no attention weight)."""
+    run = 3 * ps - 5 if aligned else 23       # tokens per label: aligned, 3 pages each, the third not full
     sizes = [1, ps, 31 * ps, 32 * ps, 33 * ps - 1, 4096 // ps * ps - 2, 70 * ps + 5, 5 * ps]
+    if aligned:                               # the new token (label 6) opens the last page of the range
+        sizes = [1, ps, 10 * run, 10 * run + 2 * ps, 11 * run - 1, 85 * run if ps == 16 else 42 * run + 10, 23 * run + 5,
+                 2 * run]
     cut = [0, 1, 1, 31, 17, 90, 200, 99]
     B = len(sizes)
     for weight in (1.0, 0.0):
@@ -469,7 +586,7 @@ def test_one_launch_observation_selects_what_the_two_kernels_select(ps, aligned,
             for r in range(7):
                 c.set_region_params(r, 0.0 if weight == 0.0 else 0.3 + 0.1 * r, 20.0, r == 0)
             for b, m in enumerate(sizes):
-                lab = (np.arange(m) // 23 % 7).astype(np.uint8)
+                lab = (np.arange(m) // run % 7).astype(np.uint8)
                 k, v = synth.kv_host(19, b, 1, 1, 0, m, lab)
                 c.append_tokens(b, lab, to_dev(k), to_dev(v), -(np.arange(m, dtype=np.int32)[::-1] // 40))
             c.calib_enable(two_kernels)
@@ -478,9 +595,13 @@ def test_one_launch_observation_selects_what_the_two_kernels_select(ps, aligned,
             out = torch.empty((B, 1, 4, 128), dtype=torch.int16, device="cuda")
             c.decode_step(B, to_dev(q), to_dev(kn), to_dev(vn), [6] * B, out)
             pages = [c.query(md.MD_QUERY_PAGES, b) for b in range(B)]
+            assert max(pages) == 4096 // ps
             ids = torch.full((B, 700), -7, dtype=torch.int32, device="cuda")
             before = c.get_state(md.MD_STATE_BLOCK_TABLE)
+            c.profile_enable(True)
             st, n_ev = c.evict([max(0, p - e) for p, e in zip(pages, cut)], ids)
+            ran = c.profile_read()
+            assert (ran["score"][1], ran["select"][1]) == (1, int(two_kernels))
             assert c.sync() == md.MD_OK
             got.append([before, torch.from_numpy(n_ev), ids] + [c.get_state(w) for w in (
                 md.MD_STATE_PAGE_SCORE, md.MD_STATE_BLOCK_TABLE, md.MD_STATE_PAGE_FILL, md.MD_STATE_SEQ_TOKENS)])
@@ -810,7 +931,9 @@ def test_capacity_and_argument_errors_are_synchronous():
     assert e.value.status == md.MD_ERR_STATE
     for key, bad in ((md.MD_DEBUG_ZERO_COPY, 2), (md.MD_DEBUG_COMBINE_OVERHEAD, -1),
                      (md.MD_DEBUG_COMBINE_OVERHEAD, 1 << 20), (md.MD_DEBUG_GRID_LIMIT, md.MD_MAX_CHUNKS - 1),
-                     (md.MD_DEBUG_FORCE_CHUNKS, md.MD_MAX_CHUNKS + 1), (99, 0)):
+                     (md.MD_DEBUG_FORCE_CHUNKS, md.MD_MAX_CHUNKS + 1), (md.MD_DEBUG_CLUSTER_FORM, 3 + 256 * 4),
+                     (md.MD_DEBUG_CLUSTER_FORM, 32 + 256 * 4), (md.MD_DEBUG_CLUSTER_FORM, 2 + 256 * 5),
+                     (md.MD_DEBUG_CLUSTER_FORM, 2 + 256 * 4 + 65536 * 2), (md.MD_DEBUG_CLUSTER_FORM, -1), (99, 0)):
         with pytest.raises(md.MemDecayError) as e:
             c.debug_set(key, bad)
         assert e.value.status == md.MD_ERR_INVALID_ARG, (key, bad)

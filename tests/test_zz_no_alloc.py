@@ -19,6 +19,7 @@ if not torch.cuda.is_available():  # pragma: no cover
 import paper_2607_10582_gb300 as md  # noqa: E402
 import synth  # noqa: E402
 from paper_2607_10582_gb300 import build as mdbuild  # noqa: E402
+from tests.attention_shapes import NOALLOC_PERSISTENT  # noqa: E402
 from tests.gpu_harness import TOL_FLOOR, TOL_O_ABS, TOL_REL, to_dev  # noqa: E402
 
 mdbuild.build()
@@ -28,12 +29,9 @@ synth.build()
 @pytest.mark.parametrize("L,Hq,ps,lengths", [
     (2, 16, 16, [900, 2500]),
     (2, 12, 32, [3000, 70, 1500]),
-    # many items and long sequences: the split that fills the grid (3 chunks
-    # per item) does not fit the fixed array, so the call takes 4; the
-    # 40-token sequence gets fewer chunks than the others
+    # many items and long sequences, one short one: clusters of 8-warp CTAs
     (16, 16, 16, [3000] * 7 + [40] + [3000] * 8),
-    # a serving batch shaped like the 3B geometry at budget: one chunk per
-    # item, no partials
+    # a serving batch shaped like the 3B geometry at budget: one CTA per item
     (36, 16, 16, [420 + 9 * i for i in range(32)]),
 ])
 def test_noalloc_matches_workspace_path_twice(L, Hq, ps, lengths):
@@ -79,12 +77,50 @@ def test_noalloc_matches_workspace_path_twice(L, Hq, ps, lengths):
     c.close()
 
 
+@pytest.mark.parametrize("L,Hq,Hkv,ps,lengths", NOALLOC_PERSISTENT)
+def test_noalloc_on_the_persistent_kernel_twice(L, Hq, Hkv, ps, lengths):
+    """The persistent kernel with the fixed array (score rows, counters, and
+    partials where an item has several chunks) against attention in 64 bits, on
+    two calls in a row: the second finds the first one's leftovers."""
+    B, P, G = len(lengths), max(lengths) // ps + 1, Hq // Hkv
+    pages = [(n + ps - 1) // ps for n in lengths]
+    NP = sum(pages)
+    g = torch.Generator(device="cuda").manual_seed(59)
+    pool = torch.randn((L, NP, Hkv, 2, ps, 128), generator=g, device="cuda").bfloat16()
+    ids = torch.randperm(NP, generator=g, device="cuda")
+    bt = torch.zeros((B, P), dtype=torch.int32, device="cuda")
+    first = 0
+    for b in range(B):
+        bt[b, :pages[b]] = ids[first:first + pages[b]]
+        first += pages[b]
+    q = torch.randn((B, L, Hq, 128), generator=g, device="cuda").bfloat16()
+    n_tok = np.array(lengths, np.int32)
+    for call in range(2):
+        out = torch.zeros((B, L, Hq, 128), dtype=torch.bfloat16, device="cuda")
+        mass = torch.zeros((L * Hkv, NP * ps), device="cuda")
+        st = md.lib().md_attend_mass_noalloc(pool.data_ptr(), bt.data_ptr(), n_tok.ctypes.data, q.data_ptr(),
+                                             out.data_ptr(), mass.data_ptr(), B, L, Hq, Hkv, ps, P, NP,
+                                             torch.cuda.current_stream().cuda_stream)
+        assert st == md.MD_OK
+        torch.cuda.synchronize()
+        for b in range(B):
+            n, pg = lengths[b], bt[b, :pages[b]].long()
+            kv = pool[:, pg].double().transpose(1, 2)                  # [L][Hkv][pages][2][ps][128]
+            k, v = (kv[:, :, :, i].reshape(L, Hkv, -1, 128)[:, :, :n] for i in (0, 1))
+            p = torch.softmax(torch.einsum("lhgd,lhnd->lhgn", q[b].double().view(L, Hkv, G, 128), k) / 128 ** 0.5, -1)
+            o = torch.einsum("lhgn,lhnd->lhgd", p, v).reshape(L, Hq, 128)
+            assert float((out[b].double() - o).abs().max()) <= TOL_O_ABS, (call, b)
+            want = p.sum(2).reshape(L * Hkv, n)
+            slots = (pg[:, None] * ps + torch.arange(ps, device="cuda")).flatten()[:n]
+            rel = ((mass[:, slots].double() - want).abs() / (want + TOL_FLOOR)).max()
+            assert float(rel) <= TOL_REL, (call, b, float(rel))
+
+
 @pytest.mark.parametrize("L,Hq,Hkv,ps,lengths", [
     (1, 16, 2, 16, [1]),
     (1, 12, 2, 32, [1703, 33]),
     (2, 16, 2, 16, [430 - 3 * i for i in range(32)]),
-    (1, 16, 2, 16, [20007 - 16 * i for i in range(8)]),      # the persistent kernel
-    (1, 8, 2, 32, [20017 - 32 * i for i in range(8)]),       # the same
+    *NOALLOC_PERSISTENT,
 ])
 @pytest.mark.parametrize("stale", [0x7FFF, 0x7F80])          # a NaN and an infinity
 def test_noalloc_ignores_what_lies_past_the_cached_tokens(L, Hq, Hkv, ps, lengths, stale):
