@@ -84,7 +84,6 @@ struct md_ctx {
   std::vector<ProfRec> pending;
   double prof_ms[N_STAGES] = {0};
   int64_t prof_n[N_STAGES] = {0};
-  std::vector<uint8_t> staging_host;
 };
 
 namespace {
@@ -511,7 +510,6 @@ size_t md::compute_layout(const md_config &c, Layout *lay) {
   L.scratch = take((size_t)MAX_GRID * 2 * L.scratch_tokens * GP * 4, 256);
   L.partials = take(L.n_items * L.chunk_stride * PARTIAL_FLOATS * 4, 256);
   L.counters = take(L.n_items * 4, 256);
-  L.evict_list = take((size_t)c.max_batch * c.max_pages_per_seq * 4, 256);
   L.staging_regions = take((size_t)c.max_pages_per_seq * ps, 256);
   L.staging_steps = take((size_t)c.max_pages_per_seq * ps * 4, 256);
   L.staging_slots = take((size_t)c.max_pages_per_seq * ps * 4, 256);
@@ -1165,7 +1163,6 @@ MD_API md_status md_evict(md_ctx *c, int batch, const int32_t *budget, int32_t *
       sel.page_score = ptr<float>(c, c->lay.page_score);
       sel.block_table = ptr<int32_t>(c, c->lay.block_table);
       sel.free_stack = ptr<int32_t>(c, c->lay.free_stack);
-      sel.evict_list = ptr<int32_t>(c, c->lay.evict_list);
       sel.user_evicted = evicted_ids_dev;
       sel.page_fill = ptr<uint8_t>(c, c->lay.page_fill);
       sel.seq_tokens = ptr<int32_t>(c, c->lay.seq_tokens);

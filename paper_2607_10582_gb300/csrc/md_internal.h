@@ -41,7 +41,7 @@ struct RegionTable {
 /* Byte offsets of every array inside the caller's workspace. */
 struct Layout {
   size_t pool, block_table, page_score, free_stack, region, a, t_ref, t_ins, window, ahat, prio, mass_acc,
-      scratch, partials, counters, evict_list, staging_regions, staging_steps, staging_slots, status,
+      scratch, partials, counters, staging_regions, staging_steps, staging_slots, status,
       calib, page_fill, seq_tokens, io_q, io_k, io_v, io_out, total;
   size_t slots, n_items;
   int scratch_tokens, chunk_stride;
@@ -241,7 +241,6 @@ struct SelectParams {
   const float *page_score;
   int32_t *block_table;
   int32_t *free_stack;
-  int32_t *evict_list;    // [max_batch][P_max] internal
   int32_t *user_evicted;  // optional [n_seqs][P_max]
   uint8_t *page_fill;     // [max_batch][P_max], compacted with the block table
   int32_t *seq_tokens;    // [max_batch], less the evicted pages' tokens

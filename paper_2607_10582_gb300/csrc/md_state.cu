@@ -570,7 +570,6 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const __grid_consta
     if (in) {
       const int id = phys[i];
       if (ev) {
-        p.evict_list[(size_t)b * p.P_max + idx_ev] = id;
         p.free_stack[base_push + idx_ev] = id;
         if (uout) uout[idx_ev] = id;
         gone += fills[i];
