@@ -826,19 +826,27 @@ md_status append_step(md_ctx *c, int batch, int l0, int L, const void *k_new, co
   return e == cudaSuccess ? MD_OK : cuda_fail(c, e, "append launch");
 }
 
-/* Whether the persistent kernel also appends a step's new tokens.  The unit
- * with a sequence's last page then fetches, patches and writes two rows, about
- * 0.3 us of a CTA's time per (sequence, layer, KV head) item, against the 2.5
- * us of a launch of its own: it pays up to 3 items per CTA (2 sequences of
- * 30,000 tokens in 36 layers, 144 items: 341.5 us, 344 with the launch; 16 of
- * 500 to 8,000 in 28, 896 items: 316 both; 12 of 1,100, 4 KV heads, 36 layers,
- * 1,728 items: 157.6 and 154.0; 256 of 300, 18,432 items: 508.5 and 479.4).
- * Region-aligned pages always take the launch: the producer reads a fill per
- * page, and telling the last page from the others there slows every page
- * (22 sequences of 4,160 tokens, 8 layers, 2 steps: 602 and 512 us). */
+/* Whether the persistent kernel also appends a step's new tokens, or follows an
+ * append launch (2.5 us).  Inside, the unit with a sequence's last page fetches,
+ * patches and writes two rows, 0.3 to 0.6 us of a CTA's time per (sequence,
+ * layer, KV head) item, and with 16-token pages the producer's test for the last
+ * page costs about 16 us per million pages.  Measured inside / apart, us:
+ *   pages of 32: 40 sequences of 1,700 tokens in 36 layers (2,880 items) 371.5 /
+ *     377.2, 40 of 6,500 1,383 / 1,385; 64 of 200 (4,608 items) 102.0 / 96.7, 256
+ *     of 100 (18,432 items) 316 / 281.
+ *   pages of 16: 16 of 1,700 (1,152 items, 123,000 pages) 165.3 / 166.0, 2 of
+ *     20,000 (180,000) 239.2 / 241.3, 12 of 6,500 (351,000) 442.0 / 439.0, 32 of
+ *     6,500 (938,000) 1,134 / 1,121; 64 of 200 (4,608 items) 106.3 / 98.7.
+ *   region-aligned pages: the producer reads a fill per page, and telling the last
+ *     page from the others there slows every page: 16 of 6,500 658 / 578 with
+ *     pages of 16, 4 of 65,000 1,419 / 1,397 with pages of 32. */
 bool append_inside(const md_ctx *c, int batch, int layers) {
-  return !c->cfg.region_aligned_pages &&
-         (long long)batch * layers * c->cfg.num_kv_heads <= 3LL * c->grid_limit;
+  if (c->cfg.region_aligned_pages) return false;
+  const long long lh = (long long)layers * c->cfg.num_kv_heads, items = batch * lh;
+  if (c->cfg.page_size == 32) return items <= 12LL * c->grid_limit;
+  long long pages = 0;
+  for (int b = 0; b < batch; ++b) pages += c->n_pages[b];
+  return items <= 4LL * c->grid_limit && pages * lh <= 200000;
 }
 
 /* Stage 1 over layers [l0, l0 + L); q/out hold q_layers layers.  With k_new

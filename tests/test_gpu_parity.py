@@ -661,19 +661,20 @@ def test_append_in_one_call_and_in_pieces(ps, aligned, runs):
 @pytest.mark.parametrize("kernel", ["cluster", "persistent", "persistent, many items"])
 def test_append_inside_attention_writes_what_the_append_kernel_writes(ps, aligned, entry, kernel):
     """Decode steps whose attention launch appends the new tokens (the cluster
-    kernel; the persistent one with contiguous pages and at most three items per
-    CTA, else it follows an append launch) leave the same pool, token state and
+    kernel; the persistent one with contiguous pages and few items per CTA, else
+    it follows an append launch) leave the same pool, token state and
     page tables, bit for bit, as steps with host buffers, whose append is always
     a launch of its own.  Lengths put the new token on the first and the last
     slot of a page, on both 16-token tiles of a 32-token page and into an empty
     sequence; region changes open pages early."""
     L, Hq, Hkv = 2, 16, 2
     lengths = [0, 1, ps - 1, ps, ps + 1, 5 * ps - 1, 33 * ps, 700]
-    if kernel == "persistent, many items":
-        lengths = lengths + [3 * i % 67 for i in range(232)]       # 960 items of the step, 480 of a layer
+    if kernel == "persistent, many items":                          # 4,000 items of the step, 500 of a layer
+        L, lengths = 8, lengths + [3 * i % 67 for i in range(242)]
     B = len(lengths)
     rng = np.random.default_rng(7)
-    caches = [md.Cache(L, Hq, Hkv, ps, B, 64, 64 * B, region_aligned_pages=aligned) for _ in range(2)]
+    pages = sum(n // ps + (40 if aligned else 12) for n in lengths) + 100
+    caches = [md.Cache(L, Hq, Hkv, ps, B, 64, pages, region_aligned_pages=aligned) for _ in range(2)]
     if kernel != "cluster":
         for c in caches:
             c.debug_set(md.MD_DEBUG_GRID_LIMIT, 128)
