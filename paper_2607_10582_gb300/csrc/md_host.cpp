@@ -834,9 +834,10 @@ md_status append_step(md_ctx *c, int batch, int l0, int L, const void *k_new, co
  *   pages of 32: 40 sequences of 1,700 tokens in 36 layers (2,880 items) 371.5 /
  *     377.2, 40 of 6,500 1,383 / 1,385; 64 of 200 (4,608 items) 102.0 / 96.7, 256
  *     of 100 (18,432 items) 316 / 281.
- *   pages of 16: 16 of 1,700 (1,152 items, 123,000 pages) 165.3 / 166.0, 2 of
- *     20,000 (180,000) 239.2 / 241.3, 12 of 6,500 (351,000) 442.0 / 439.0, 32 of
- *     6,500 (938,000) 1,134 / 1,121; 64 of 200 (4,608 items) 106.3 / 98.7.
+ *   pages of 16: 12 of 1,700 (864 items, 92,000 pages) 126.2 / 127.2, 14 of up to
+ *     3,211 in 24 layers (120,000) 180.3 / 176.4, 12 of 6,500 (351,000) 442.0 /
+ *     439.0, 32 of 6,500 (938,000) 1,134 / 1,121; 64 of 200 (4,608 items) 106.3 /
+ *     98.7.
  *   region-aligned pages: the producer reads a fill per page, and telling the last
  *     page from the others there slows every page: 16 of 6,500 658 / 578 with
  *     pages of 16, 4 of 65,000 1,419 / 1,397 with pages of 32. */
@@ -846,7 +847,7 @@ bool append_inside(const md_ctx *c, int batch, int layers) {
   if (c->cfg.page_size == 32) return items <= 12LL * c->grid_limit;
   long long pages = 0;
   for (int b = 0; b < batch; ++b) pages += c->n_pages[b];
-  return items <= 4LL * c->grid_limit && pages * lh <= 200000;
+  return items <= 4LL * c->grid_limit && pages * lh <= 100000;
 }
 
 /* Stage 1 over layers [l0, l0 + L); q/out hold q_layers layers.  With k_new
