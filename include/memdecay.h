@@ -289,9 +289,9 @@ md_status md_load_state(md_ctx *ctx, const void *src_dev, const void *host_blob)
 
 /* Per-stage GPU time, from CUDA events recorded around each launch while
  * enabled.  Stages: 0 append, 1 attention (stage 1), 2 window fold,
- * 3 score + page reduce (stages 2-3), 4 select + compact (stage 4).  Decode
- * steps with device buffers append inside the attention launch (counted there),
- * and short sequences are scored and selected in one launch (counted as 3).
+ * 3 score + page reduce (stages 2-3), 4 select + compact (stage 4).  Most
+ * decode steps with device buffers append inside the attention launch (counted
+ * there), and short sequences are scored and selected in one launch (counted as 3).
  * md_profile_read synchronises the stream and returns, for each stage, the
  * summed milliseconds and the number of launches since enabling.  Each event
  * pair keeps consecutive kernels from overlapping (about 2 us per event on a
@@ -395,7 +395,8 @@ md_status md_calib_fit(const double *mass_sum, const int64_t *count, int n_bucke
  *
  *   kv_pool_dev      bf16 [L][num_phys_pages][Hkv][2][page_size][128]: for
  *                    each (layer, page, KV head) the page's K rows then its V
- *                    rows (md_decode_step's pool layout; 16-byte aligned)
+ *                    rows (md_decode_step's pool layout; 16-byte aligned);
+ *                    slots past a sequence's tokens may hold anything
  *   block_table_dev  int32 [batch][max_pages_per_seq] physical page ids
  *   n_tokens_host    [batch] cached tokens per sequence (host), each >= 1 and
  *                    at most max_pages_per_seq * page_size

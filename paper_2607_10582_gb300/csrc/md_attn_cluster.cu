@@ -1,6 +1,7 @@
-/* Stage 1 for launches that fit the chip in one wave: the same attention and
- * exact mass as attn_mass_kernel, with one CTA per chunk of a (sequence,
- * layer, KV head) item and the item's chunks in one thread-block cluster.
+/* Stage 1 for launches of one to a few waves of CTAs (cluster_plan draws the
+ * line): the same attention and exact mass as attn_mass_kernel, with one CTA per
+ * chunk of a (sequence, layer, KV head) item and the item's chunks in one
+ * thread-block cluster.
  *
  * What bounds these launches is latency, not HBM: a layer of a 32-sequence
  * batch at a 430-token budget reads 12 MB (1.8 us at 6.8 TB/s).  The
@@ -495,9 +496,10 @@ static int seq_tiles(const AttnBase &p, int b) {
 
 /* Which kernel, and how many CTAs and warps per item: the least of these costs
  * in us, fitted to 57 launch shapes timed on a GB300 in every form (1 to 64
- * sequences of 128 to 30,000 tokens, one layer and whole steps): on average
- * 1% above the best form, and 1.48 times as fast as the persistent kernel
- * alone.  n: 16-token tiles per warp, N: CTAs, hbm: the K/V bytes at 6.8 TB/s.
+ * sequences of 128 to 30,000 tokens, one layer and whole steps).  Over 48 shapes
+ * (1 to 64 sequences of 30 to 100,000 tokens) its choice takes 1.4% longer than
+ * the best form of each, 14% at worst (5 sequences of 700 tokens in 36 layers,
+ * 33.0 and 29.1), and the persistent kernel alone 34% longer than its choice.  n: 16-token tiles per warp, N: CTAs, hbm: the K/V bytes at 6.8 TB/s.
  *   One wave (the N CTAs run at once): the CTA's time (launch chain, prologue
  *     and merge in `base`, 0.65 or 0.74 per tile of its warps; the cluster's
  *     exchange raises `base`) or HBM's, and 0.006 N.  One layer of 1 x 430
