@@ -274,6 +274,8 @@ class Cache:
         sp = None
         if insert_steps is not None:
             steps, sp = _host(insert_steps, np.int32)
+            if steps.size < regs.size:
+                raise MemDecayError(MD_ERR_INVALID_ARG, f"{steps.size} insertion steps for {regs.size} labels")
         return self._check(lib().md_append_tokens(self.h, seq, len(regs), rp, sp, _ptr(k), _ptr(v)))
 
     def decode_step(self, batch: int, q, k_new, v_new, new_regions, out):

@@ -66,3 +66,15 @@ def test_labels_fewer_than_the_batch_are_refused(calls, regs):
         assert e.value.status == md.MD_ERR_INVALID_ARG
     with pytest.raises(md.MemDecayError, match="null handle"):      # layers after the first read no labels
         c.decode_layer(1, 2, None, None, None, regs, None)
+
+
+def test_fewer_insertion_steps_than_labels_are_refused():
+    """The library reads one insertion step per label."""
+    c = object.__new__(md.Cache)
+    c.h = None
+    for steps in ([0], np.zeros(1, np.int32), []):
+        with pytest.raises(md.MemDecayError, match="insertion steps") as e:
+            c.append_tokens(0, [5, 6], None, None, steps)
+        assert e.value.status == md.MD_ERR_INVALID_ARG
+    with pytest.raises(md.MemDecayError, match="null handle"):
+        c.append_tokens(0, [5, 6], None, None, [0, 0])
